@@ -129,15 +129,15 @@ int pfmp_op_destroy(pfmp_op* op);
 /* sum over odd sites of log det A(x) (host scalar; synchronises).                    */
 int pfmp_op_logdet(pfmp_op* op, double* logdet_oo);
 /* Threads per output site of the stencil kernels of this operator for one arithmetic
- * (prec = PFMP_F64, PFMP_F32 or PFMP_DF): 1, 2, 4 or 8.  Splitting a site's 8 hop terms
- * across threads adds parallelism where the kernel is latency- or ALU-bound (small
- * lattices, FP64, double-float).  Results differ only by summation order.  The default
- * comes from pfmp_op_create (a fixed rule on precision and lattice size, so runs are
- * reproducible); pfmp_op_get_split reads it.                                         */
+ * (prec = PFMP_F64, PFMP_F32 or PFMP_DF): 1, 2, 4 or 8.  2, 4 and 8 split a site's 8 hop
+ * terms across that many threads of a warp; 1 (the default) leaves the kernel to the
+ * library's own rule on precision and lattice size (fixed, so runs are reproducible): one
+ * thread per site, or a block-shared site for FP64, double-float and small FP32 lattices.
+ * Results differ only by summation order.                                            */
 int pfmp_op_set_split(pfmp_op* op, int prec, int nsplit);
 int pfmp_op_get_split(pfmp_op* op, int prec, int* nsplit);
-/* Threads per block of this operator's stencil kernels (32, 64, 96 or 128; default from
- * pfmp_op_create: the lattice's sites per parity spread over the SMs in whole waves).  */
+/* Threads per block of this operator's one-thread-per-site and split-site stencil kernels
+ * (32, 64, 96 or 128; default 128).                                                    */
 int pfmp_op_set_block(pfmp_op* op, int threads);
 
 /* Wilson hop restricted to one parity: out (parity out_parity) = H_{out,in} in; with

@@ -13,6 +13,7 @@
 // cross terms, renormalised.
 #pragma once
 #include "fields.cuh"
+#include "mad.cuh"
 
 namespace pfmp {
 
@@ -54,6 +55,8 @@ __device__ __forceinline__ df operator*(df x, df y) {
   e = __fmaf_rn(x.lo, y.hi, e);
   return df_fast_two_sum(p, e);
 }
+
+__device__ __forceinline__ df mad(df x, df y, df z) { return z + x * y; }
 
 template <>
 struct Prec<2> {  // double-float, used only inside the library (the true residual)

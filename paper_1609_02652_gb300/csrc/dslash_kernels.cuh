@@ -4,10 +4,11 @@
 // adjoint) pair, so that the heavy template instantiations compile in parallel;
 // dslash.h declares what they export and dslash.cu dispatches on run-time arguments.
 //
-// One thread per output site.  Each thread spin-projects its 8 neighbours to
-// two-component half spinors (the projectors (1 -+ g_mu) have rank 2), multiplies by
-// the link (FP32: 12-real links, third row rebuilt in registers), and rebuilds the
-// four-component result.  Two fused epilogues make M-hat a two-kernel operation:
+// FP32 and FP16 storage: one thread per output site (k_hop).  Each thread spin-projects its
+// 8 neighbours to two-component half spinors (the projectors (1 -+ g_mu) have rank 2),
+// multiplies by the link (12-real links, third row rebuilt in registers), and rebuilds the
+// four-component result.  FP64, double-float and FP32 on small lattices: several threads
+// per site (hop_tile.cuh).  Two fused epilogues make M-hat a two-kernel operation:
 //   EPI_CLOV  out = C (H in)            (odd sites: C = A_oo^{-1})
 //   EPI_XPAY  out = C x + coef (H in)   (even sites: C = A_ee, x the local input), with
 //             an optional grid reduction of ||out||^2 feeding the CG scalars.
@@ -17,16 +18,7 @@
 #include "dslash.h"
 #include "dfloat.cuh"
 #include "hop.cuh"
-
-#ifndef HOP_MINB_F32
-#define HOP_MINB_F32 7
-#endif
-#ifndef HOP_MINB_H16
-#define HOP_MINB_H16 6
-#endif
-#ifndef HOP_MINB_F64
-#define HOP_MINB_F64 1
-#endif
+#include "hop_tile.cuh"
 
 namespace pfmp {
 
@@ -34,21 +26,11 @@ namespace pfmp {
 // stencil is bound by memory latency, so more warps in flight pay even at the cost of a
 // few spilled registers (FP32, 32^3x64: 0.85 -> 0.89 of the copy bandwidth at 7 blocks).
 // The FP16-storage stencil does more arithmetic per byte and runs best with a few more
-// registers (K at 32^3x64: 97.4 us per launch at 7 blocks, 93.1 at 6 or 5, 103 at 8);
-// FP64 and double-float keep the compiler's choice (a bound of 3 blocks made the rolled
-// double-float stencil 7-18% slower).
+// registers (K at 32^3x64: 97.4 us per launch at 7 blocks, 93.1 at 6 or 5, 103 at 8).
 template <int PREC>
 constexpr int hop_min_blocks() {
-  return PREC == PFMP_F32 ? HOP_MINB_F32 : PREC == PFMP_H16 ? HOP_MINB_H16 : PREC == PFMP_F64 ? HOP_MINB_F64 : 1;
-}
-
-// Double-float arithmetic takes the rolled stencil: unrolled, its ~18k instructions per
-// thread stall on instruction fetch (ncu at 16^3x32: ~10 "no instruction" stall cycles
-// per issue, 13% of the FP32 pipe); rolled, a K application is 2.5-2.9x faster.  FP64 is
-// bound by GB300's FP64 rate and runs slower rolled (+28%), so it stays unrolled.
-template <int PREC>
-__host__ __device__ constexpr bool hop_rolled() {
-  return PREC == PREC_DF;
+  static_assert(PREC == PFMP_F32 || PREC == PFMP_H16, "FP64 and double-float: hop_tile.cuh");
+  return PREC == PFMP_F32 ? 7 : 6;
 }
 
 template <int PREC, bool DAG, int EPI, bool REDUCE>
@@ -58,9 +40,7 @@ __global__ void __launch_bounds__(128, hop_min_blocks<PREC>()) k_hop(HopParams<P
   double nrm[1] = {0.0};
   if (cb < a.g.Vh) {
     Spinor<typename Prec<PREC>::real> out;
-    if constexpr (hop_rolled<PREC>())
-      out = hop_site_rolled<PREC, DAG, EPI>(a, cb);
-    else if constexpr (PREC == PFMP_H16)
+    if constexpr (PREC == PFMP_H16)
       out = hop_site_h16<DAG, EPI>(a, cb);
     else
       out = hop_site<PREC, DAG, EPI>(a, cb);
@@ -135,7 +115,14 @@ void launch(const HopParams<PREC>& a, pfmp_op* op) {
       case 2: k_hop_split<PREC, DAG, EPI, RED, 2><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
       case 4: k_hop_split<PREC, DAG, EPI, RED, 4><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
       case 8: k_hop_split<PREC, DAG, EPI, RED, 8><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
-      default: k_hop<PREC, DAG, EPI, RED><<<nblocks(a.g.Vh, bs), bs, 0, c->stream>>>(a); break;
+      default:
+        if constexpr (PREC == PFMP_F32) {
+          if (!hop_shared_f32(a.g.Vh)) {
+            k_hop<PREC, DAG, EPI, RED><<<nblocks(a.g.Vh, bs), bs, 0, c->stream>>>(a);
+            break;
+          }
+        }
+        launch_shared<PREC, DAG, EPI, RED>(a, c->stream);
     }
   }
   PFMP_CHECK_LAUNCH();
