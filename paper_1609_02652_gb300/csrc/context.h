@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <complex>
+#include <functional>
 #include <vector>
 
 #include "pfmp_internal.cuh"
@@ -95,7 +96,7 @@ struct pfmp_op {
     const void* key[4] = {nullptr, nullptr, nullptr, nullptr};
     int chunk = 0;
     long long kernels = 0;  // kernel nodes in the graph (for the launch counter)
-  } graph[4];
+  } graph[6];               // CG chunks by precision, then the multi-shift chunks
   cudaStream_t cap = nullptr;
   pfmp::MSWork* ms = nullptr;  // multi-shift workspace (grown on demand)
   void* fgcr = nullptr;         // FGCR workspace (kept between solves), freed by fgcr_free
@@ -206,6 +207,12 @@ void poly_product(pfmp_op* op, const std::vector<std::complex<double>>& z, doubl
 
 // probe.cu: measured FMA throughput (TFLOP/s) of the FP64 or FP32 pipe
 double fma_rate(pfmp_ctx* c, int prec);
+
+// slots of pfmp_op::graph beyond the CG's (indexed by precision)
+constexpr int kGraphMs64 = 4, kGraphMs32 = 5;
+// replay the chunk that `launch` enqueues on the context's stream as a CUDA graph, captured
+// (on op->cap) when the slot holds another key or chunk length
+void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch);
 
 // solver.cu
 int solve(pfmp_op* op, int method, double tol, int max_iter, double delta, int check_every, void* x,

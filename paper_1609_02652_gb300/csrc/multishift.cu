@@ -9,9 +9,11 @@
 //   x_s += alpha_s p_s,  p_s = zeta_s' r + beta_s p_s,
 // where a, b are the seed CG's alpha, beta and ^- marks the previous iteration.  All
 // scalars live on the device (FP64); one iteration is K (the reduction finisher writes
-// a), the per-shift scalars, the seed residual (whose finisher writes b, the per-shift
-// coefficients and which shifts have converged), and ONE pass that updates x_s and p_s
-// of every shift still running and the seed direction.  A shift whose residual
+// a), the seed residual (whose last block writes b and, one thread per shift, the shifts'
+// coefficients and which of them have converged) and the seed direction.  The shifts'
+// vectors wait: the residuals of up to kMsBlock iterations are kept, and ONE pass then
+// carries every shift still running through all of them, so that its x_s and p_s cross
+// memory once per block instead of once per iteration.  A shift whose residual
 // |zeta_s| |r| is below tol |b| takes this iteration's x update and then stops: the
 // large shifts of a Chebyshev filter converge in a fraction of the seed's iterations,
 // and their vectors leave the memory traffic.  The loop ends when every shift has
@@ -29,6 +31,7 @@
 // (stable_order), which keeps every partial product within a few orders of magnitude of
 // the final one (in index order the partial products of P_64 reach 1e11 times it, and
 // the rounding of each factor is amplified accordingly).
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -38,17 +41,20 @@
 
 namespace pfmp {
 
+constexpr int kMsBlock = 8;  // iterations per pass over the shifts' vectors
+constexpr int kMsUpdX = 1, kMsUpdP = 2;
 struct MSShift {
   double2 sigma;
-  double2 zeta_prev, zeta, zeta_next;
-  double2 alpha;   // x_s += alpha p_s
-  double2 beta;    // p_s = zeta_next r + beta p_s
-  int active;      // takes part in this iteration
-  int keep;        // still running after it (its direction is updated)
+  double2 zeta, zeta_next;  // of the previous iteration and of this one
+  int keep;                 // still running after this iteration
+  // the block's iterations: x_s += alpha p_s (kMsUpdX), p_s = zeta r + beta p_s (kMsUpdP)
+  double2 alpha[kMsBlock], zn[kMsBlock], beta[kMsBlock];
+  int upd[kMsBlock];
 };
 struct MSSeed {
   double alpha_prev, beta_prev;
-  int nact;        // shifts active this iteration, listed in act[]
+  int nact;        // shifts active in the block's first iteration, listed in act[]
+  int count;       // iterations of the block that ran
 };
 
 __device__ __forceinline__ double2 cm(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
@@ -61,14 +67,16 @@ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ double2 cs(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
 
 // complex words of a vector field: double2 = one complex number, float4 = two
-__device__ __forceinline__ double2 axpy_c(double2 a, double2 x, double2 y) { return cadd(y, cm(a, x)); }
+__device__ __forceinline__ double2 axpy_c(double2 a, double2 x, double2 y) {
+  return make_double2(fma(-a.y, x.y, fma(a.x, x.x, y.x)), fma(a.y, x.x, fma(a.x, x.y, y.y)));
+}
 __device__ __forceinline__ float4 axpy_c(double2 a, float4 x, float4 y) {
   const float ar = (float)a.x, ai = (float)a.y;
   return make_float4(y.x + ar * x.x - ai * x.y, y.y + ar * x.y + ai * x.x, y.z + ar * x.z - ai * x.w,
                      y.w + ar * x.w + ai * x.z);
 }
 // a x + b y
-__device__ __forceinline__ double2 axpby_c(double2 a, double2 x, double2 b, double2 y) { return cadd(cm(a, x), cm(b, y)); }
+__device__ __forceinline__ double2 axpby_c(double2 a, double2 x, double2 b, double2 y) { return axpy_c(a, x, cm(b, y)); }
 __device__ __forceinline__ float4 axpby_c(double2 a, float4 x, double2 b, float4 y) {
   const float ar = (float)a.x, ai = (float)a.y, br = (float)b.x, bi = (float)b.y;
   return make_float4(ar * x.x - ai * x.y + br * y.x - bi * y.y, ar * x.y + ai * x.x + br * y.y + bi * y.x,
@@ -80,95 +88,204 @@ __device__ __forceinline__ float4 sub_real(float4 r, double ad, float4 q) {
   return make_float4(r.x - a * q.x, r.y - a * q.y, r.z - a * q.z, r.w - a * q.w);
 }
 __device__ __forceinline__ double nrm(double2 v) { return v.x * v.x + v.y * v.y; }
-__device__ __forceinline__ double nrm(float4 v) { return (double)(v.x * v.x + v.y * v.y) + (double)(v.z * v.z + v.w * v.w); }
+// |v|^2 added to a thread's running sum
+struct NormSum64 {
+  double t = 0.0;
+  __device__ __forceinline__ void add(double2 v) { t += nrm(v); }
+  __device__ __forceinline__ double value() const { return t; }
+};
+struct NormSum32 {
+  PairSum t;
+  __device__ __forceinline__ void add(float4 v) {
+    t.add(v.x * v.x + v.y * v.y);
+    t.add(v.z * v.z + v.w * v.w);
+  }
+  __device__ __forceinline__ double value() const { return t.value(); }
+};
+template <typename V>
+struct NormOf {
+  using type = NormSum64;
+};
+template <>
+struct NormOf<float4> {
+  using type = NormSum32;
+};
 __device__ __forceinline__ double2 xpby_real(double2 r, double b, double2 p) { return make_double2(r.x + b * p.x, r.y + b * p.y); }
 __device__ __forceinline__ float4 xpby_real(float4 r, double bd, float4 p) {
   const float b = (float)bd;
   return make_float4(r.x + b * p.x, r.y + b * p.y, r.z + b * p.z, r.w + b * p.w);
 }
 
-// zeta_next and alpha_s of every active shift from the seed's alpha (just computed) and
-// the previous alpha, beta
-__global__ void k_ms_alpha(MSShift* sh, int ns, const CGScalars* s, const MSSeed* sd) {
-  if (s->done) return;
-  const int i = threadIdx.x + blockIdx.x * blockDim.x;
-  if (i >= ns || !sh[i].active) return;
-  MSShift v = sh[i];
-  const double a = s->alpha, ap = sd->alpha_prev, bp = sd->beta_prev;
-  const double2 one_as = make_double2(1.0 + a * v.sigma.x, a * v.sigma.y);
-  const double2 den = cadd(cs(ap, cm(v.zeta_prev, one_as)), cs(a * bp, csub(v.zeta_prev, v.zeta)));
-  v.zeta_next = cdiv(cs(ap, cm(v.zeta, v.zeta_prev)), den);
-  v.alpha = cs(a, cdiv(v.zeta_next, v.zeta));
-  sh[i].zeta_next = v.zeta_next;
-  sh[i].alpha = v.alpha;
-}
-
-// seed residual r -= alpha Ap, |r|^2; finisher: beta, rr, iter, the shifts' direction
-// coefficients, which shifts keep running (|zeta_s'|^2 |r|^2 >= stop), done when none
+// seed residual r = r_prev - alpha Ap, |r|^2 (r, r_prev: neighbouring slots of the block's
+// residuals; this is iteration `slot` of the block).  The last block then takes one thread
+// per shift: the zetas move on, zeta_next and alpha_s from the seed's alpha and the previous
+// alpha, beta, the direction coefficients, and whether the shift keeps running
+// (|zeta_s'|^2 |r|^2 >= stop); the solve is done when none does.  (One thread doing this for
+// every shift in turn cost 10-25 us an iteration, FP64 divisions in a serial chain: the
+// kernel at 24^3x48 with 13 shifts 41 -> 27 us.)
 template <typename V>
-__global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ Ap, long n, ReduceBuf rb, CGScalars* s, MSSeed* sd,
-                       MSShift* sh, int ns) {
-  if (s->done) return;
-  const double al = s->alpha;
-  double v[1] = {0.0};
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const V rr = sub_real(r[i], al, Ap[i]);
-    r[i] = rr;
-    v[0] += nrm(rr);
+__global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V* __restrict__ Ap, long n, ReduceBuf rb,
+                       CGScalars* s, MSSeed* sd, MSShift* sh, int ns, int* act, int slot) {
+  if (s->done) {  // a block that starts after the end has no iterations
+    if (slot == 0 && blockIdx.x == 0 && threadIdx.x == 0) sd->count = 0;
+    return;
   }
+  const double al = s->alpha;
+  typename NormOf<V>::type acc;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    const V rr = sub_real(r_prev[i], al, Ap[i]);
+    r[i] = rr;
+    acc.add(rr);
+  }
+  double v[1] = {acc.value()};
   double t[1];
-  if (grid_sum<1>(v, rb, t)) {
-    const double beta = t[0] / s->rr;
+  if (!grid_sum_last<1>(v, rb, t)) return;
+  __shared__ int wcount[kBlock / 32];
+  const double rr0 = s->rr, stop = s->stop_rr, beta = t[0] / rr0;
+  const double ap = sd->alpha_prev, bp = sd->beta_prev;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int any = 0, listed = 0;
+  for (int k0 = 0; k0 < ns; k0 += blockDim.x) {
+    const int k = k0 + threadIdx.x;
+    int on = 0, keep = 0;
+    if (k < ns) {
+      MSShift& S = sh[k];
+      on = S.keep;
+      if (on) {
+        const double2 zp = S.zeta, z = S.zeta_next;  // this iteration's zeta_prev and zeta
+        const double2 one_as = make_double2(1.0 + al * S.sigma.x, al * S.sigma.y);
+        const double2 den = cadd(cs(ap, cm(zp, one_as)), cs(al * bp, csub(zp, z)));
+        const double2 zn = cdiv(cs(ap, cm(z, zp)), den);
+        const double2 q = cdiv(zn, z);
+        keep = nrm(zn) * t[0] >= stop;
+        S.zeta = z;
+        S.zeta_next = zn;
+        S.keep = keep;
+        S.alpha[slot] = cs(al, q);
+        S.zn[slot] = zn;
+        S.beta[slot] = cs(beta, cm(q, q));
+      }
+      S.upd[slot] = on ? (keep ? kMsUpdX | kMsUpdP : kMsUpdX) : 0;
+    }
+    if (slot == 0) {  // list the block's shifts in ascending order
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (lane == 0) wcount[warp] = __popc(m);
+      __syncthreads();
+      int at = listed + __popc(m & ((1u << lane) - 1));
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        if (w < warp) at += wcount[w];
+        listed += wcount[w];
+      }
+      if (on) act[at] = k;
+    }
+    any |= __syncthreads_or(keep);
+  }
+  if (threadIdx.x == 0) {
+    sd->alpha_prev = al;
+    sd->beta_prev = beta;
+    if (slot == 0) sd->nact = listed;
+    sd->count = slot + 1;
     s->beta = beta;
     s->rr = t[0];
     s->iter += 1;
-    sd->alpha_prev = al;
-    sd->beta_prev = beta;
-    bool any = false;
-    for (int k = 0; k < ns; ++k) {
-      if (!sh[k].active) continue;
-      const double2 q = cdiv(sh[k].zeta_next, sh[k].zeta);
-      sh[k].beta = cs(beta, cm(q, q));
-      const int keep = nrm(sh[k].zeta_next) * t[0] >= s->stop_rr;
-      sh[k].keep = keep;
-      any = any || keep;
-    }
-    if (!any || !(t[0] == t[0])) s->done_next = 1;
+    if (!any || !(t[0] == t[0])) s->done = 1;
   }
 }
 
-// x_s += alpha_s p_s and p_s = zeta_s' r + beta_s p_s for the active shifts (the
-// direction only for those that keep running), the seed p = r + beta p; the finisher
-// rotates the zetas and the active set
+// seed direction p = r + beta p
 template <typename V>
-__global__ void k_ms_xp(V* const* x, V* const* p, V* __restrict__ pseed, const V* __restrict__ r, MSShift* sh,
-                        int ns, const int* act, MSSeed* sd, long n, ReduceBuf rb, CGScalars* s) {
+__global__ void k_ms_p(V* __restrict__ p, const V* __restrict__ r, long n, const CGScalars* s) {
   if (s->done) return;
   const double be = s->beta;
-  const int na = sd->nact;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const V rr = r[i];
-    for (int j = 0; j < na; ++j) {
-      const int k = act[j];
-      const V pk = p[k][i];
-      x[k][i] = axpy_c(sh[k].alpha, pk, x[k][i]);
-      if (sh[k].keep) p[k][i] = axpby_c(sh[k].zeta_next, rr, sh[k].beta, pk);
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+    p[i] = xpby_real(r[i], be, p[i]);
+}
+
+// coefficients and fields of one shift in the arithmetic of its vectors
+template <typename V>
+struct MSCoef;
+template <>
+struct MSCoef<double2> {
+  using C = double2;
+  static __device__ __forceinline__ C make(double2 a) { return a; }
+};
+template <>
+struct MSCoef<float4> {
+  using C = float2;
+  static __device__ __forceinline__ C make(double2 a) { return make_float2((float)a.x, (float)a.y); }
+};
+__device__ __forceinline__ float4 axpy_c(float2 a, float4 x, float4 y) {
+  return make_float4(y.x + a.x * x.x - a.y * x.y, y.y + a.x * x.y + a.y * x.x, y.z + a.x * x.z - a.y * x.w,
+                     y.w + a.x * x.w + a.y * x.z);
+}
+__device__ __forceinline__ float4 axpby_c(float2 a, float4 x, float2 b, float4 y) {
+  return make_float4(a.x * x.x - a.y * x.y + b.x * y.x - b.y * y.y, a.x * x.y + a.y * x.x + b.x * y.y + b.y * y.x,
+                     a.x * x.z - a.y * x.w + b.x * y.z - b.y * y.w, a.x * x.w + a.y * x.z + b.x * y.w + b.y * y.z);
+}
+
+// The shifts' pass: for every shift listed, the block's iterations in order,
+// x_s += alpha_s p_s and p_s = zeta_s' r + beta_s p_s (the direction only while the shift
+// keeps running), with r[slot] the residual of iteration `slot`.  Bound by the copy
+// bandwidth: two vectors read and two written per shift and kMsBlock iterations (24^3x48,
+// 13 FP32 shifts: 265 us an iteration at 0.97 of the bandwidth when the pass ran every
+// iteration, 391 us for eight now).  Block row blockIdx.y takes every gridDim.y-th shift of the list
+// (small lattices: the shifts are the parallelism).  The coefficients are converted once
+// per block and held in shared memory.
+constexpr int kMsTile = 16;
+template <typename V>
+struct MSRing {
+  V* r[kMsBlock];
+};
+template <typename V>
+__global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRing<V> ring, const MSShift* __restrict__ sh,
+                                                  const int* __restrict__ act, const MSSeed* sd, long n) {
+  using C = typename MSCoef<V>::C;
+  const int cnt = sd->count;
+  if (cnt == 0) return;
+  __shared__ V* sx[kMsTile];
+  __shared__ V* sp[kMsTile];
+  __shared__ C ca[kMsTile][kMsBlock], cz[kMsTile][kMsBlock], cb[kMsTile][kMsBlock];
+  __shared__ int up[kMsTile][kMsBlock];
+  const int na = sd->nact, G = gridDim.y;
+  const int mine = na > (int)blockIdx.y ? (na - 1 - (int)blockIdx.y) / G + 1 : 0;  // shifts of this row
+  const long step = (long)gridDim.x * blockDim.x, i0 = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  for (int j0 = 0; j0 < mine; j0 += kMsTile) {
+    const int m = mine - j0 < kMsTile ? mine - j0 : kMsTile;
+    __syncthreads();
+    for (int q = threadIdx.x; q < m * kMsBlock; q += blockDim.x) {
+      const int j = q / kMsBlock, b = q % kMsBlock, k = act[(j0 + j) * G + blockIdx.y];
+      if (b == 0) {
+        sx[j] = x[k];
+        sp[j] = p[k];
+      }
+      up[j][b] = b < cnt ? sh[k].upd[b] : 0;
+      ca[j][b] = MSCoef<V>::make(sh[k].alpha[b]);
+      cz[j][b] = MSCoef<V>::make(sh[k].zn[b]);
+      cb[j][b] = MSCoef<V>::make(sh[k].beta[b]);
     }
-    pseed[i] = xpby_real(rr, be, pseed[i]);
-  }
-  double v[1] = {0.0}, t[1];
-  if (grid_sum<1>(v, rb, t)) {
-    int m = 0;
-    int* a = const_cast<int*>(act);
-    for (int k = 0; k < ns; ++k) {
-      if (!sh[k].active) continue;
-      sh[k].zeta_prev = sh[k].zeta;
-      sh[k].zeta = sh[k].zeta_next;
-      sh[k].active = sh[k].keep;
-      if (sh[k].keep) a[m++] = k;
+    __syncthreads();
+    for (long i = i0; i < n; i += step) {
+      V rr[kMsBlock];
+#pragma unroll
+      for (int b = 0; b < kMsBlock; ++b)
+        if (b < cnt) rr[b] = ring.r[b][i];
+#pragma unroll 2
+      for (int j = 0; j < m; ++j) {
+        V pk = sp[j][i], xk = sx[j][i];
+        int last = 0;
+#pragma unroll
+        for (int b = 0; b < kMsBlock; ++b) {
+          const int u = up[j][b];
+          if (u) {
+            xk = axpy_c(ca[j][b], pk, xk);
+            if (u & kMsUpdP) pk = axpby_c(cz[j][b], rr[b], cb[j][b], pk);
+            last = u;
+          }
+        }
+        sx[j][i] = xk;
+        if (last & kMsUpdP) sp[j][i] = pk;
+      }
     }
-    sd->nact = m;
-    s->done = s->done_next;
   }
 }
 
@@ -210,8 +327,11 @@ struct MSWork {
   MSSeed* d_seed = nullptr;
   int* d_act = nullptr;
   int cap = 0;
+  std::vector<void*> ring[2];  // the block's residuals, FP64 and FP32
   ~MSWork() {
     for (auto q : p) dev_free(q);
+    for (auto& v : ring)
+      for (auto q : v) dev_free(q);
     dev_free(d_x);
     dev_free(d_p);
     dev_free(d_sh);
@@ -220,10 +340,16 @@ struct MSWork {
   }
 };
 
-static MSWork& ms_work(pfmp_op* op, int ns) {
+static MSWork& ms_work(pfmp_op* op, int ns, int prec) {
   if (!op->ms) op->ms = new MSWork();
   MSWork& w = *op->ms;
   if (w.cap < ns) {
+    // a captured chunk holds the arrays that are replaced here
+    for (int g : {kGraphMs64, kGraphMs32})
+      if (op->graph[g].exec) {
+        cudaGraphExecDestroy(op->graph[g].exec);
+        op->graph[g].exec = nullptr;
+      }
     while ((int)w.p.size() < ns) w.p.push_back((double2*)dev_alloc(spinor_bytes(op->ctx->g, PFMP_F64)));
     dev_free(w.d_x);
     dev_free(w.d_p);
@@ -236,6 +362,8 @@ static MSWork& ms_work(pfmp_op* op, int ns) {
     if (!w.d_seed) w.d_seed = (MSSeed*)dev_alloc(sizeof(MSSeed));
     w.cap = ns;
   }
+  auto& ring = w.ring[prec == PFMP_F64 ? 0 : 1];
+  while ((int)ring.size() < kMsBlock) ring.push_back(dev_alloc(spinor_bytes(op->ctx->g, prec)));
   return w;
 }
 
@@ -245,17 +373,33 @@ void ms_work_free(pfmp_op* op) {
 }
 
 template <typename V>
-static void ms_iteration(pfmp_op* op, int prec, MSWork& w, int ns, void* r, void* pseed, void* Ap, long n) {
+static void ms_chunk(pfmp_op* op, int prec, MSWork& w, int ns, void* pseed, void* Ap, long n, int chunk) {
   pfmp_ctx* c = op->ctx;
-  kop(op, prec, Ap, pseed, &op->scal->pAp, op->scal);
-  k_ms_alpha<<<(ns + 127) / 128, 128, 0, c->stream>>>(w.d_sh, ns, op->scal, w.d_seed);
-  PFMP_CHECK_LAUNCH();
-  k_ms_r<V><<<ms_grid(n), kBlock, 0, c->stream>>>((V*)r, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh, ns);
-  PFMP_CHECK_LAUNCH();
-  k_ms_xp<V><<<ms_grid(n), kBlock, 0, c->stream>>>((V* const*)w.d_x, (V* const*)w.d_p, (V*)pseed, (const V*)r,
-                                                   w.d_sh, ns, w.d_act, w.d_seed, n, c->rb, op->scal);
-  PFMP_CHECK_LAUNCH();
+  MSRing<V> ring;
+  for (int b = 0; b < kMsBlock; ++b) ring.r[b] = (V*)w.ring[prec == PFMP_F64 ? 0 : 1][b];
+  // rows of shifts until the pass has about four blocks per SM
+  const int nb = ms_grid(n), rows = std::max(1, std::min(ns, 152 * 4 / nb));
+  for (int k = 0; k < chunk; ++k) {
+    const int slot = k % kMsBlock;
+    kop(op, prec, Ap, pseed, &op->scal->pAp, op->scal);
+    // the residual before a chunk is in the last slot (every chunk but the last is whole blocks)
+    const V* prev = ring.r[slot == 0 ? kMsBlock - 1 : slot - 1];
+    k_ms_r<V><<<nb, kBlock, 0, c->stream>>>(ring.r[slot], prev, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh, ns,
+                                            w.d_act, slot);
+    PFMP_CHECK_LAUNCH();
+    k_ms_p<V><<<nb, kBlock, 0, c->stream>>>((V*)pseed, ring.r[slot], n, op->scal);
+    PFMP_CHECK_LAUNCH();
+    if (slot == kMsBlock - 1 || k == chunk - 1) {
+      k_ms_xp<V><<<dim3(nb, rows), kBlock, 0, c->stream>>>((V* const*)w.d_x, (V* const*)w.d_p, ring, w.d_sh, w.d_act,
+                                                           w.d_seed, n);
+      PFMP_CHECK_LAUNCH();
+    }
+  }
 }
+
+// Up to this many sites per parity the kernels of an iteration are shorter than the
+// host takes to launch them, and a chunk is replayed as a CUDA graph (as the CG's).
+constexpr int kMsGraphMax = 32768;
 
 // x[k] = (K + sigma_k)^{-1} b in FP64 or FP32 (x, b of precision prec).  Returns the
 // status; iterations, K applications and (FP64, on request) the largest true residual.
@@ -275,7 +419,8 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
                  "multi-shift CG: a real negative shift can make K + sigma singular");
   }
   if (check <= 0) check = 8;
-  MSWork& w = ms_work(op, ns);
+  check = (check + kMsBlock - 1) / kMsBlock * kMsBlock;  // whole blocks between host checks
+  MSWork& w = ms_work(op, ns, prec);
   const size_t bytes = spinor_bytes(c->g, prec);
   const long n = words(c->g, prec);
   blas_norm2(c, prec, b, c->d_sums);
@@ -288,7 +433,7 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
   for (int k = 0; k < ns; ++k) blas_zero(c, prec, x[k]);
   if (bb == 0.0) return PFMP_OK;
   PFMP_REQUIRE(std::isfinite(bb), PFMP_E_NAN, "right-hand side is not finite");
-  void* r = prec == PFMP_F64 ? (void*)op->cg64[0] : (void*)op->cg32[0];
+  void* r = w.ring[prec == PFMP_F64 ? 0 : 1][kMsBlock - 1];
   void* pseed = prec == PFMP_F64 ? (void*)op->cg64[1] : (void*)op->cg32[1];
   void* Ap = prec == PFMP_F64 ? (void*)op->cg64[2] : (void*)op->cg32[2];
   PFMP_CUDA(cudaMemcpyAsync(r, b, bytes, cudaMemcpyDeviceToDevice, c->stream));
@@ -303,15 +448,15 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
     PFMP_CUDA(cudaMemcpyAsync(w.p[k], b, bytes, cudaMemcpyDeviceToDevice, c->stream));
     MSShift s{};
     s.sigma = make_double2(sigma[k].real(), sigma[k].imag());
-    s.zeta_prev = s.zeta = s.zeta_next = make_double2(1.0, 0.0);
-    s.active = s.keep = 1;
+    s.zeta = s.zeta_next = make_double2(1.0, 0.0);
+    s.keep = 1;
     hs[k] = s;
   }
   PFMP_CUDA(cudaMemcpyAsync(w.d_x, hx.data(), ns * sizeof(void*), cudaMemcpyHostToDevice, c->stream));
   PFMP_CUDA(cudaMemcpyAsync(w.d_p, hp.data(), ns * sizeof(void*), cudaMemcpyHostToDevice, c->stream));
   PFMP_CUDA(cudaMemcpyAsync(w.d_sh, hs.data(), ns * sizeof(MSShift), cudaMemcpyHostToDevice, c->stream));
   PFMP_CUDA(cudaMemcpyAsync(w.d_act, act.data(), ns * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  MSSeed sd{1.0, 0.0, ns};
+  MSSeed sd{1.0, 0.0, ns, 0};
   PFMP_CUDA(cudaMemcpyAsync(w.d_seed, &sd, sizeof(MSSeed), cudaMemcpyHostToDevice, c->stream));
   CGScalars* h = op->h_scal;
   *h = CGScalars{};
@@ -322,11 +467,17 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
   const long long kapply0 = op->kapply;  // queued iterations after convergence do no work
   while (done < max_iter) {
     const int chunk = check < max_iter - done ? check : max_iter - done;
-    for (int k = 0; k < chunk; ++k) {
+    auto launch = [&]() {
       if (prec == PFMP_F64)
-        ms_iteration<double2>(op, prec, w, ns, r, pseed, Ap, n);
+        ms_chunk<double2>(op, prec, w, ns, pseed, Ap, n, chunk);
       else
-        ms_iteration<float4>(op, prec, w, ns, r, pseed, Ap, n);
+        ms_chunk<float4>(op, prec, w, ns, pseed, Ap, n, chunk);
+    };
+    if (c->g.Vh <= kMsGraphMax && !c->prof.on) {
+      const void* key[4] = {w.d_sh, w.d_x, w.d_p, (const void*)(intptr_t)ns};
+      run_graph(op, op->graph[prec == PFMP_F64 ? kGraphMs64 : kGraphMs32], key, chunk, launch);
+    } else {
+      launch();
     }
     PFMP_CUDA(cudaMemcpyAsync(h, op->scal, sizeof(CGScalars), cudaMemcpyDeviceToHost, c->stream));
     PFMP_CUDA(cudaStreamSynchronize(c->stream));

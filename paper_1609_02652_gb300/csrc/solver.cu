@@ -82,23 +82,11 @@ static void launch_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void*
   }
 }
 
-// One chunk of CG iterations.  Without kernel profiling the chunk is captured once into
-// a CUDA graph (6 kernels per iteration, 4 for FP32; all parameters fixed: the scalars
+// A chunk of iterations, captured once into a CUDA graph (all parameters fixed: the scalars
 // live on the device) and replayed on the context's stream, which removes the per-launch
 // host cost.
-// K applications are counted by run_cg from the iterations the device actually ran (the
-// queued kernels of a converged chunk return at once), so the count kop keeps while the
-// chunk is launched or captured is put back afterwards.
-static void run_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void* Ap, int chunk) {
+void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch) {
   pfmp_ctx* c = op->ctx;
-  const long long kapply0 = op->kapply;
-  if (c->prof.on) {
-    launch_chunk(op, prec, x, r, p, Ap, chunk);
-    op->kapply = kapply0;
-    return;
-  }
-  pfmp_op::Graph& G = op->graph[prec];
-  const void* key[4] = {x, r, p, Ap};
   bool hit = G.exec && G.chunk == chunk;
   for (int k = 0; k < 4 && hit; ++k) hit = G.key[k] == key[k];
   if (!hit) {
@@ -109,11 +97,12 @@ static void run_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void* Ap
     if (!op->cap) PFMP_CUDA(cudaStreamCreateWithFlags(&op->cap, cudaStreamNonBlocking));
     cudaStream_t keep = c->stream;
     cudaGraph_t graph = nullptr;
+    const long long kapply0 = op->kapply;
     PFMP_CUDA(cudaStreamBeginCapture(op->cap, cudaStreamCaptureModeThreadLocal));
     c->stream = op->cap;
     const long long n0 = launch_count();
     try {
-      launch_chunk(op, prec, x, r, p, Ap, chunk);
+      launch();
     } catch (...) {
       c->stream = keep;
       cudaStreamEndCapture(op->cap, &graph);
@@ -133,6 +122,22 @@ static void run_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void* Ap
   }
   PFMP_CUDA(cudaGraphLaunch(G.exec, c->stream));
   count_launches(G.kernels);
+}
+
+// One chunk of CG iterations (6 kernels per iteration, 4 for the fused FP32 one), as a graph
+// unless kernels are being profiled.  K applications are counted by run_cg from the
+// iterations the device actually ran (the queued kernels of a converged chunk return at
+// once), so the count kop keeps while the chunk is launched or captured is put back.
+static void run_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void* Ap, int chunk) {
+  auto launch = [&]() { launch_chunk(op, prec, x, r, p, Ap, chunk); };
+  if (op->ctx->prof.on) {
+    const long long kapply0 = op->kapply;
+    launch();
+    op->kapply = kapply0;
+    return;
+  }
+  const void* key[4] = {x, r, p, Ap};
+  run_graph(op, op->graph[prec], key, chunk, launch);
 }
 
 // run the device CG loop (prec) until `done` or the iteration cap; returns iterations
