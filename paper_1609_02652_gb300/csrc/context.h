@@ -61,6 +61,7 @@ struct pfmp_ctx {
   long fmunu_version = -1;   // gauge_version it was computed for
   int fmunu_prec = PFMP_F64; // arithmetic it was computed in
   float* hc32 = nullptr;     // FP32 copy of a clover insertion for the FP32 clover force (on demand)
+  void* clov_d[2] = {nullptr, nullptr};  // the clover force's D matrices, FP64 and FP32 (on demand)
 };
 
 struct pfmp_op {
@@ -168,6 +169,7 @@ struct DerivSet {
 constexpr int kMaxDerivSets = 8;
 struct DerivBatch {
   int n = 0;
+  double c_common = 1.0;  // c_hop of every contraction where they agree, else 1 (set per launch)
   DerivSet s[kMaxDerivSets];
 };
 // F and Hc += every contraction of the batch, one launch per force kernel: the

@@ -297,6 +297,7 @@ void ctx_destroy(pfmp_ctx* c) {
   dev_free(c->canon);
   dev_free(c->fmunu);
   dev_free(c->hc32);
+  for (auto q : c->clov_d) dev_free(q);
   if (c->h_sums) cudaFreeHost(c->h_sums);
   delete c;
 }
