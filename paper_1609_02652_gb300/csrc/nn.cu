@@ -542,8 +542,7 @@ struct pfmp_nn {
   bool tc = false;               // use it in nn_apply
   bool packed = false;           // Bp holds the current weights
   std::vector<void*> Bp;         // packed FP16 operand per layer
-  std::vector<void*> act16;      // FP16 scaled inputs of each layer
-  void* z16 = nullptr;           // last layer: FP16 per-direction mixed outputs [9][12][V]
+  void* act16[2] = {nullptr, nullptr};  // FP16 scaled activations between the layers, in turn
   float* sigma = nullptr;        // device scalar: 1 / rms of the network input
   int* err = nullptr;            // device error flag of the tensor-core kernel
   long long id = 0;              // unique per network (keys the FGCR cycle graphs)
@@ -556,21 +555,21 @@ static size_t csz(const pfmp_nn* N) { return N->prec == PFMP_F64 ? sizeof(double
 bool nn_tc_supported(int cin, int cout);
 size_t nn_tc_packed_bytes(int cin, int cout);
 void nn_tc_pack(pfmp_ctx* c, int cin, int cout, const void* W, void* Bp);
+size_t nn_tc_act_bytes(const Geom& g);
 void nn_tc_scale(pfmp_ctx* c, const void* in_even_f32, float* sigma_dev, const int* skip);
-void nn_tc_layer(pfmp_ctx* c, int cin, int cout, bool last, const void* Bp, const void* in, void* out,
-                 const float* sigma, int* err, const int* skip);
-void nn_tc_embed(pfmp_ctx* c, const void* in_even_f32, float* sigma, void* act16, const int* skip, const double* rr);
-void nn_tc_last(pfmp_ctx* c, const void* Bp, const void* in, void* z16, void* out_even_f32, const float* sigma,
-                int* err, const int* skip);
-void nn_tc_init();
+void nn_tc_first(pfmp_ctx* c, const void* Bp, const void* in, void* act, float* sigma, const double* rr, int* err,
+                 const int* skip);
+void nn_tc_hidden(pfmp_ctx* c, const void* Bp, const void* in, void* out, int* err, const int* skip);
+void nn_tc_last(pfmp_ctx* c, const void* Bp, const void* in, void* z, void* out, float* sigma, int* err, const int* skip);
+int nn_tc_init();
 
 void nn_destroy(pfmp_nn* N) {
   if (!N) return;
-  for (auto* vec : {&N->W, &N->gW, &N->m, &N->v, &N->act, &N->Bp, &N->act16})
+  for (auto* vec : {&N->W, &N->gW, &N->m, &N->v, &N->act, &N->Bp})
     for (auto p : *vec) dev_free(p);
   dev_free(N->sigma);
   dev_free(N->err);
-  dev_free(N->z16);
+  for (auto p : N->act16) dev_free(p);
   dev_free(N->gbuf[0]);
   dev_free(N->gbuf[1]);
   dev_free(N->target);
@@ -611,9 +610,8 @@ pfmp_nn* nn_create(pfmp_ctx* c, int nl, const int* ch, int prec) {
     if (all) {  // every layer on the tensor cores (1 -> 8, 8 -> 8 ..., 8 -> 1)
       for (int l = 0; l < nl; ++l) {
         N->Bp.push_back(dev_alloc(nn_tc_packed_bytes(ch[l], ch[l + 1])));
-        N->act16.push_back(dev_alloc((size_t)ch[l] * 12 * c->g.V * 4));
       }
-      N->z16 = dev_alloc((size_t)9 * 12 * c->g.V * 4);
+      for (auto& p : N->act16) p = dev_alloc(nn_tc_act_bytes(c->g));
       N->tc = true;
       N->sigma = (float*)dev_alloc(sizeof(float));
       N->err = (int*)dev_alloc(sizeof(int));
@@ -715,12 +713,10 @@ static void forward_tc(pfmp_nn* N, void* out, const void* in, const int* skip, c
   pfmp_ctx* c = N->ctx;
   const int L = (int)N->W.size();
   if (!rr) nn_tc_scale(c, in, N->sigma, skip);
-  nn_tc_embed(c, in, N->sigma, N->act16[0], skip, rr);
-  for (int l = 0; l < L - 1; ++l)
-    nn_tc_layer(c, N->ch[l], N->ch[l + 1], false, N->Bp[l], N->act16[l], N->act16[l + 1], N->sigma, N->err, skip);
-  // the last layer mixes channels at each site first and transports after (the colour
-  // transport commutes with the spin/channel weights), on even sites only
-  nn_tc_last(c, N->Bp[L - 1], N->act16[L - 1], N->z16, out, N->sigma, N->err, skip);
+  nn_tc_first(c, N->Bp[0], in, N->act16[0], N->sigma, rr, N->err, skip);
+  for (int l = 1; l < L - 1; ++l) nn_tc_hidden(c, N->Bp[l], N->act16[(l - 1) & 1], N->act16[l & 1], N->err, skip);
+  // the last layer's mixed channels take the other buffer, whose contents have been used
+  nn_tc_last(c, N->Bp[L - 1], N->act16[L & 1], N->act16[(L & 1) ^ 1], out, N->sigma, N->err, skip);
 }
 
 template <typename T>

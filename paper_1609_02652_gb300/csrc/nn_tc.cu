@@ -1,69 +1,98 @@
-// Tensor-core forward layers of the gauge-covariant network (C_in -> C_out channels with
-// C_in, C_out in {1, 8}).
+// Tensor-core inference of the gauge-covariant network 1 -> 8 -> ... -> 8 -> 1.
 //
-// The layer is a dense contraction per site and colour:
+// A layer is a dense contraction per site and colour:
 //   y[o][a](x, c) = sum_d sum_i sum_b W_d[o][i][a][b] t_d[i][b](x, c),
 // t_d = the input channel parallel-transported from the neighbour in direction d (the
 // site itself, four forward and four backward hops, fermion boundary factor included).
-// As a real GEMM per colour: rows = 128 sites of a tile (M = 128, one TMEM lane each),
-// K = 9 directions x C_in channels x 4 spins x (re, im), N = C_out x 4 spins x (re, im)
+// As a real GEMM per colour: rows = 128 sites of one parity (M = 128, one TMEM lane each),
+// K = directions x C_in channels x 4 spins x (re, im), N = C_out x 4 spins x (re, im)
 // (padded to 16), with B = [[Re W, -Im W], [Im W, Re W]] so that the complex product
 // comes out in (re, im) column pairs.  Operands are FP16, the accumulator FP32 in
-// tensor memory.  K is consumed in stages: one direction per stage (K = 8 C_in), or for
-// C_in = 1 four directions per stage (K = 32, the last stage three quarters zero).
+// tensor memory; the transport itself is FP32 (links and products).
 //
-// Activations between the layers are FP16 complex [C][12][V], scaled by sigma = 1/rms of
-// the network input so that FP16 keeps its precision (the network is linear; the last
-// layer writes FP32 divided by sigma).  The directions are taken in the order site, +x,
-// -x, +y, -y, +z, -z, +t, -t so that consecutive stages read overlapping neighbours.
+// The network input lives on even sites and its output is read there, so two of the layers
+// are half empty:
+//   first (1 -> 8)   even sites see only their own input, odd sites only their eight
+//                    neighbours: one stage per tile, straight from the FP32 input field
+//                    (k_nn_single<true>; nine direction slots of 8 columns, K = 16 or 80)
+//   hidden (8 -> 8)  nine stages of K = 64, one direction each (k_nn_hidden)
+//   last (8 -> 1)    the channels are mixed at every site first (the colour transport commutes
+//                    with the weights): z_0 = W_0 a on even sites, z_d = W_d a for the eight
+//                    hops on odd sites (k_nn_single<false>, K = 64), then out(x) = z_0(x) +
+//                    sum_d U_d(x) z_d(x + d) on even sites in FP32 (k_nn_last)
+// Activations between the layers are FP16, scaled by sigma = 1/rms of the network input so
+// that FP16 keeps its precision (the network is linear; the last layer divides by sigma).
+// Layout [parity][block of 32 sites][channel][12][32 sites], a complex number per word: the
+// 96 words of a site lie at constant offsets (one address per neighbour) and a warp's 32
+// neighbours touch one or two blocks.
 //
-// One CTA per SM loops over tiles of 128 sites.  Per stage, 512 threads (four per
-// site) gather and transport the inputs (FP32 links) into a K-major shared-memory tile per
-// colour (no-swizzle canonical layout: 8-row x 16-byte core matrices, K-adjacent cores
-// 128 bytes apart, 8-row groups 16 K bytes apart), then one thread issues the
-// tcgen05.mma instructions of the three colours and commits them to an mbarrier; the
-// A tiles are double-buffered so that the gather of stage s + 1 overlaps the MMAs of
-// stage s.  The packed weights of all stages (72 KB for 8 -> 8) stay in shared memory,
-// brought in by bulk TMA copies.  The epilogue reads the accumulators with
-// tcgen05.ld (lane = site) and writes the output activations.
+// What bounds k_nn_hidden: instruction issue and the L2 gather (3.5 KB per site), not the
+// tensor pipe.  The earlier kernel ran load -> transport -> barrier in lockstep (issue slots
+// half idle, 196 us at 16^3x32).  Now eight warps gather (two threads per site, four channels
+// each) and a ninth issues the MMAs: they meet only on mbarriers, a channel pair's registers
+// are refilled for the next stage as soon as it is transported, two channels share one packed
+// FP32 instruction (fma.rn.f32x2), the site's own stage is copied bit for bit, and a tile's
+// accumulators are read two stages into the next tile (two sets in tensor memory).
+// The rounding points and the order of the transport's products are fixed (transport_pair):
+// an FP16 activation turns a change in the last bit of its FP32 value into one of 2^-11.
+// One application of [1, 8, 8, 8, 1] at 16^3x32: 568 -> 319 us; per kernel (before): scale 9 (9),
+// first layer 28 (61 with the embedding), hidden 115 (196), mixing 16 (39), last 12 (40).
+// Tried and slower: sixteen gathering warps of 128 registers (150 us per hidden layer: the
+// links' work doubles), eight warps with 255 registers that issue the MMAs themselves (155).
+//
 // Every mbarrier wait is bounded; on a timeout the kernel raises a device error flag,
 // waits (bounded) for the work it has in flight, frees its tensor memory and returns.
 #include <cuda_fp16.h>
 
-#include <cstdlib>
+#include <algorithm>
+#include <type_traits>
 
 #include "context.h"
 #include "fields.cuh"
+#include "mad.cuh"
 
 namespace pfmp {
 namespace tc {
 
 constexpr int kM = 128;        // sites per tile = TMEM lanes
-constexpr int kThreads = 512;  // four threads per site in the gather
-// COUT = 9 marks the local mixing of the last layer: z_d = sum_i W_d[0][i] a_i at every
-// site for the nine directions d (no gather; the transport follows in k_last_stencil)
-template <int CIN, int COUT>
-struct Shape {
-  static constexpr bool LOCAL = COUT == 9;
-  static constexpr int NST = LOCAL ? 1 : (CIN == 1 ? 3 : 9);  // K stages
-  static constexpr int DPS = CIN == 1 ? 4 : 1;        // directions per stage
-  static constexpr int K = CIN == 1 ? 32 : 8 * CIN;   // reals per stage
-  static constexpr int N = (8 * COUT + 15) / 16 * 16;  // output reals per colour (padded to 16)
-  static constexpr int A_TILE = kM * K * 2;
-  static constexpr int A_BUF = 3 * A_TILE;
-  static constexpr int B_ST = N * K * 2;
+constexpr int kGather = 256;   // gathering threads: two per site
+constexpr int kWords = 96;     // complex words of a site's activations (8 channels)
+constexpr int kSiteBlock = 32; // sites per activation block
+constexpr int kCh = 8;         // hidden channels
+constexpr int kK = 8 * kCh;    // reals of one stage
+constexpr int kATile = kM * kK * 2;  // A tile of one colour
+constexpr int kABuf = 3 * kATile;
+
+struct Hidden {
+  static constexpr int NST = 9;
+  static constexpr int N = 64;
+  static constexpr int B_ST = N * kK * 2;
   static constexpr int B_ALL = NST * B_ST;
-  static constexpr int SMEM = B_ALL + 2 * A_BUF;
-  static constexpr int TMEM_COLS = 3 * N <= 32 ? 32 : (3 * N <= 64 ? 64 : (3 * N <= 128 ? 128 : 256));
-  static constexpr uint32_t SBO = 16 * K;  // bytes between 8-row groups
-  static_assert(3 * N <= 256 && N % 16 == 0 && K % 16 == 0, "tile shape");
-  static_assert(CIN == 1 || CIN == 8, "the gather splits 8 channels over four threads per site");
+  static constexpr int SMEM = B_ALL + 2 * kABuf;
+  static constexpr int SET = 3 * N;  // TMEM columns of one accumulator set
+  static constexpr int TMEM_COLS = 512;  // two sets
+  static_assert(2 * SET <= TMEM_COLS && SMEM <= 227 * 1024, "tile shape");
+};
+// the one-stage layers: A of 8 SLOTS columns (first: the site, eight hops, padding; last: the
+// channels), B for the even and the odd sites
+template <bool FIRST>
+struct Single {
+  static constexpr int KD = FIRST ? 80 : kK;        // columns of the A tile
+  static constexpr int K_EVEN = FIRST ? 16 : kK;    // of them used on even sites
+  static constexpr int N_EVEN = FIRST ? 64 : 16, N_ODD = 64;
+  static constexpr int B_EVEN = N_EVEN * K_EVEN * 2, B_ODD = N_ODD * KD * 2;
+  static constexpr int B_ALL = B_EVEN + B_ODD;
+  static constexpr int A_TILE = kM * KD * 2;
+  static constexpr int SMEM = B_ALL + 3 * A_TILE;
+  static constexpr int TMEM_COLS = 256;  // two blocks per SM share the 512 columns
 };
 
 // stage order of the nine directions (0 = site, 1 + mu = forward, 5 + mu = backward)
 __host__ __device__ __forceinline__ int dir_of(int i) {
   return i == 0 ? 0 : (i & 1 ? 1 + (i >> 1) : 5 + ((i - 1) >> 1));
 }
+
+__host__ __device__ __forceinline__ size_t act_blocks(int Vh) { return (size_t)(Vh + kSiteBlock - 1) / kSiteBlock; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -83,20 +112,55 @@ __host__ __device__ constexpr uint32_t idesc(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// non-blocking polls, backing off after the first thousand; gives up after ~2^20 polls
-// (a fraction of a second) so that a lost completion cannot hang the GPU
+// bounded wait: polls that suspend for at most a microsecond each, given up after half a second
+// (a lost completion cannot hang the GPU)
+__device__ __forceinline__ unsigned long long timer_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(1000u)
+      : "memory");
+  return ok;
+}
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int it = 0; it < (1 << 20); ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (it > 1024) __nanosleep(64);
-  }
+  if (mbar_poll(bar, parity)) return true;
+  const unsigned long long t0 = timer_ns();
+  while (timer_ns() - t0 < 500000000ull)
+    if (mbar_poll(bar, parity)) return true;
   return false;
+}
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "r"(cols));
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_free(uint32_t tmem, uint32_t cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -125,35 +189,45 @@ __device__ __forceinline__ uint32_t pack_h2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// packed B operand of one layer: [NST][N x K] FP16, each stage a K-major canonical tile
-template <int CIN, int COUT>
-__global__ void k_pack_b(const float2* __restrict__ W, __half* __restrict__ B) {
-  using S = Shape<CIN, COUT>;
+// ---------------------------------------------------------------- packed weights
+// [[Re w, -Im w], [Im w, Re w]] at (row n = output reals, column k = input reals)
+__device__ __forceinline__ float b_entry(const float2 w, int n, int k) {
+  const int ro = n & 1, ri = k & 1;
+  return ro == ri ? w.x : (ro == 0 ? -w.y : w.y);
+}
+// hidden: nine stages [64 x 64], each a K-major canonical tile
+__global__ void k_pack_hidden(const float2* __restrict__ W, __half* __restrict__ B) {
+  using S = Hidden;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= S::NST * S::N * S::K) return;
-  const int st = i / (S::N * S::K), rem = i % (S::N * S::K);
-  const int n = rem / S::K, k = rem % S::K;
-  const int di = st * S::DPS + (CIN == 1 ? (k >> 3) : 0);
-  const int ic = CIN == 1 ? 0 : (k >> 3);
-  const int o = n >> 3, a = (n >> 1) & 3, ro = n & 1;
-  const int b = (k >> 1) & 3, ri = k & 1;
+  if (i >= S::NST * S::N * kK) return;
+  const int st = i / (S::N * kK), n = i % (S::N * kK) / kK, k = i % kK;
+  const int o = n >> 3, a = (n >> 1) & 3, ic = k >> 3, b = (k >> 1) & 3;
+  const float v = b_entry(W[(((size_t)dir_of(st) * kCh + o) * kCh + ic) * 16 + a * 4 + b], n, k);
+  B[(size_t)st * (S::B_ST / 2) + kmajor(n, k, kK) / 2] = __float2half_rn(v);
+}
+// first: column slot j holds direction dir_of(j) (slot 9 is padding, as is slot 1 on even
+// sites); last: the rows of even sites are the direction 0 (rows 8.. padding), those of odd
+// sites the hops 1..8
+template <bool FIRST>
+__global__ void k_pack_single(const float2* __restrict__ W, __half* __restrict__ B) {
+  using S = Single<FIRST>;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= S::B_ALL / 2) return;
+  const bool even = i < S::B_EVEN / 2;
+  const int K = even ? S::K_EVEN : S::KD, e = even ? i : i - S::B_EVEN / 2;
+  const int n = e / K, k = e % K;
+  const int o = n >> 3, a = (n >> 1) & 3, j = k >> 3, b = (k >> 1) & 3;
   float v = 0.f;
-  if (S::LOCAL) {  // output block o is the direction d of the single output channel
-    if (o < 9) {
-      const float2 w = W[((size_t)o * CIN + ic) * 16 + a * 4 + b];
-      v = ro == ri ? w.x : (ro == 0 ? -w.y : w.y);
-    }
+  if (FIRST) {
+    if (even ? j == 0 : j < 9) v = b_entry(W[((size_t)dir_of(j) * kCh + o) * 16 + a * 4 + b], n, k);
   } else {
-    const int d = di < 9 ? dir_of(di) : 9;
-    if (d < 9 && o < COUT) {
-      const float2 w = W[(((size_t)d * COUT + o) * CIN + ic) * 16 + a * 4 + b];
-      v = ro == ri ? w.x : (ro == 0 ? -w.y : w.y);
-    }
+    if (!even || o == 0) v = b_entry(W[((size_t)(even ? 0 : 1 + o) * kCh + j) * 16 + a * 4 + b], n, k);
   }
-  B[(size_t)st * (S::B_ST / 2) + kmajor(n, k, S::K) / 2] = __float2half_rn(v);
+  B[(even ? 0 : S::B_EVEN / 2) + kmajor(n, k, K) / 2] = __float2half_rn(v);
 }
 
 // sigma = sqrt(n) / |in| (1 for a zero input) of an even FP32 field
+__device__ __forceinline__ float sigma_of(double rr, int Vh) { return rr > 0 ? (float)sqrt(24.0 * Vh / rr) : 1.0f; }
 __global__ void k_rms_scale(const float4* __restrict__ in, int Vh, ReduceBuf rb, float* sigma,
                             const int* __restrict__ skip) {
   if (skip && *skip) return;
@@ -165,651 +239,574 @@ __global__ void k_rms_scale(const float4* __restrict__ in, int Vh, ReduceBuf rb,
   }
   double s[1] = {(double)st};
   double t[1];
-  if (grid_sum<1>(s, rb, t)) *sigma = t[0] > 0 ? (float)sqrt(24.0 * Vh / t[0]) : 1.0f;
+  if (grid_sum<1>(s, rb, t)) *sigma = sigma_of(t[0], Vh);
 }
 
-// neighbour, link and boundary factor of direction d at site x: the input of the item
-// is f U a(y) (forward hop), f U^dag a(y) (backward hop) or a(x) (d = 0)
-struct Hop {
-  size_t sy;
-  float f;
-  int kind;
-  Mat3<float> U;
+// ---------------------------------------------------------------- transport
+// a site of the tile: coordinates and lexicographic index
+struct Site {
+  int x[4], lex;
 };
-__device__ __forceinline__ void make_hop(const Geom& g, const float4* __restrict__ U32, const int x[4], int d,
-                                         Hop& h) {
-  h.kind = d == 0 ? 0 : (d <= 4 ? 1 : 2);
-  const int mu = d == 0 ? 0 : (d - 1) & 3;
-  int y[4] = {x[0], x[1], x[2], x[3]};
-  h.f = 1.0f;
-  if (h.kind == 1) {
-    y[mu] = y[mu] + 1 == g.L[mu] ? 0 : y[mu] + 1;
-    if (mu == 3 && x[3] == g.L[3] - 1) h.f *= (float)g.bc_t;
-    const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-    load_link(h.U, U32 + (size_t)((p * 4 + mu) * 3) * g.Vh, cb_index(g, x), g.Vh);
-  } else if (h.kind == 2) {
-    y[mu] = y[mu] == 0 ? g.L[mu] - 1 : y[mu] - 1;
-    if (mu == 3 && x[3] == 0) h.f *= (float)g.bc_t;
-    const int p = (y[0] + y[1] + y[2] + y[3]) & 1;
-    Mat3<float> L;
-    load_link(L, U32 + (size_t)((p * 4 + mu) * 3) * g.Vh, cb_index(g, y), g.Vh);
-    h.U = dagger(L);
-  }
-  h.sy = (size_t)lex_index(g, y);
+__device__ __forceinline__ Site site_at(const Geom& g, int cb, int p) {
+  Site s;
+  cb_coords(g, cb, p, s.x);
+  s.lex = lex_index(g, s.x);
+  return s;
 }
-
-// channel-major activations act[C][12][V] (half2 complex): component k of channel ic at
-// site sy; the threads of a warp (consecutive sites) read consecutive words
-template <int C>
-__device__ __forceinline__ void load_channel(const __half2* __restrict__ in, size_t V, size_t sy, int ic,
-                                             cplx<float> v[4][3]) {
+// checkerboard index of the neighbour of stage i (1..8: +x, -x, +y, ...) and whether the hop
+// crosses the time boundary
+__device__ __forceinline__ int hop_site(const Geom& g, const Site& s, int i, bool& edge) {
+  const int mu = (i - 1) >> 1;
+  const bool fwd = i & 1;
+  int xm = s.x[0], Lm = g.L[0], stride = 1;
+  if (mu >= 1) xm = s.x[1], stride = g.L[0], Lm = g.L[1];
+  if (mu >= 2) xm = s.x[2], stride *= g.L[1], Lm = g.L[2];
+  if (mu == 3) xm = s.x[3], stride *= g.L[2], Lm = g.L[3];
+  const bool wrap = xm == (fwd ? Lm - 1 : 0);
+  edge = wrap && mu == 3;
+  const int step = wrap ? -(Lm - 1) * stride : stride;
+  return (s.lex + (fwd ? step : -step)) >> 1;
+}
+// rows 0 and 1 of the link of stage i seen from the site cb (index n: its neighbour)
+__device__ __forceinline__ void load_link_raw(float4 l[3], const float4* __restrict__ U32, int Vh, int p, int i, int cb,
+                                              int n) {
+  const int mu = (i - 1) >> 1;
+  const bool fwd = i & 1;
+  const float4* f = U32 + (size_t)(((fwd ? p : 1 - p) * 4 + mu) * 3) * Vh + (fwd ? cb : n);
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp)
+  for (int k = 0; k < 3; ++k) l[k] = __ldg(f + (size_t)k * Vh);
+}
+// the transport matrix f U or f U^dag, f = bc on hops across the time boundary, else 1
+template <bool FWD>
+__device__ __forceinline__ Mat3<float> transport_matrix(const float4 l[3], bool edge, float bc) {
+  Mat3<float> L, M;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    L.m[(2 * k) / 3][(2 * k) % 3] = mk(l[k].x, l[k].y);
+    L.m[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(l[k].z, l[k].w);
+  }
+  reconstruct_row2(L);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float2 w = __half22float2(__ldg(in + ((size_t)ic * 12 + sp * 3 + c) * V + sy));
-      v[sp][c] = mk(w.x, w.y);
+      M.m[r][c] = FWD ? L.m[r][c] : conj(L.m[c][r]);
     }
+  if (edge) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) M.m[r][c] = bc * M.m[r][c];
+  }
+  return M;
 }
 
-// transport one channel and store it (FP16) at column col of the three colour tiles
-template <int K>
-__device__ __forceinline__ void store_channel(const Hop& h, const cplx<float> v[4][3], bool live, unsigned char* A,
-                                              int row, int col, int a_tile) {
-  cplx<float> t[4][3];
-  if (live) {
-    if (h.kind) {
+// two FP32 numbers in one register pair: the same operation on both in one instruction
+typedef unsigned long long f2x;
+__device__ __forceinline__ f2x f2x_mk(float a, float b) {
+  f2x r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2x_get(f2x v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2x f2x_mul(f2x a, f2x b) {
+  f2x r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2x f2x_fma(f2x a, f2x b, f2x c) {
+  f2x r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2x f2x_add(f2x a, f2x b) {
+  f2x r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+struct Mat3x2 {  // a transport matrix for two channels at once
+  f2x re[3][3], im[3][3], ni[3][3];
+};
+__device__ __forceinline__ Mat3x2 pair_matrix(const Mat3<float>& M) {
+  Mat3x2 P;
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
+  for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-          t[sp][r] = h.f * (h.U.m[r][0] * v[sp][0] + h.U.m[r][1] * v[sp][1] + h.U.m[r][2] * v[sp][2]);
-    } else {
-#pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int r = 0; r < 3; ++r) t[sp][r] = h.f * v[sp][r];
+    for (int c = 0; c < 3; ++c) {
+      P.re[r][c] = f2x_mk(M.m[r][c].re, M.m[r][c].re);
+      P.im[r][c] = f2x_mk(M.m[r][c].im, M.m[r][c].im);
+      P.ni[r][c] = f2x_mk(-M.m[r][c].im, -M.m[r][c].im);
     }
-  } else {
+  return P;
+}
+// M v for two spinor colour vectors at once (v0, v1: three FP16 colours each), back to FP16.
+// Each complex product is rounded by itself (real part fma(re, re, -(im im)), imaginary part
+// fma(im, re, re im)) and the three are added in order.
+__device__ __forceinline__ void transport_pair(const Mat3x2& P, const uint32_t v0[3], const uint32_t v1[3], uint32_t o0[3],
+                                               uint32_t o1[3]) {
+  f2x re[3], im[3];
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-      for (int r = 0; r < 3; ++r) t[sp][r] = mk(0.f, 0.f);
+  for (int c = 0; c < 3; ++c) {
+    const float2 a = h2_to_f2(v0[c]), b = h2_to_f2(v1[c]);
+    re[c] = f2x_mk(a.x, b.x);
+    im[c] = f2x_mk(a.y, b.y);
   }
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    uint4 q;
-    q.x = pack_h2(t[0][r].re, t[0][r].im);
-    q.y = pack_h2(t[1][r].re, t[1][r].im);
-    q.z = pack_h2(t[2][r].re, t[2][r].im);
-    q.w = pack_h2(t[3][r].re, t[3][r].im);
-    *reinterpret_cast<uint4*>(A + r * a_tile + kmajor(row, col, K)) = q;
+    f2x x, y;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const f2x px = f2x_fma(P.re[r][c], re[c], f2x_mul(P.ni[r][c], im[c]));
+      const f2x py = f2x_fma(P.im[r][c], re[c], f2x_mul(P.re[r][c], im[c]));
+      x = c == 0 ? px : f2x_add(x, px);
+      y = c == 0 ? py : f2x_add(y, py);
+    }
+    const float2 xr = f2x_get(x), yi = f2x_get(y);
+    o0[r] = pack_h2(xr.x, yi.x);
+    o1[r] = pack_h2(xr.y, yi.y);
+  }
+}
+// the 12 words (spin, colour) of a spinor as 16-byte rows of the three colour tiles
+__device__ __forceinline__ void store_row(unsigned char* A, int a_tile, uint32_t at, const uint32_t w[12]) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r) *reinterpret_cast<uint4*>(A + r * a_tile + at) = make_uint4(w[r], w[3 + r], w[6 + r], w[9 + r]);
+}
+
+// first word of site c of parity q
+__device__ __forceinline__ size_t act_at(int q, int c, size_t nb32) {
+  return ((size_t)q * nb32 + c / kSiteBlock) * (kWords * kSiteBlock) + c % kSiteBlock;
+}
+
+// accumulators -> FP16 activations: TMEM lanes 32 (warp % 4) .., output channels 4 grp .. 4 grp
+// + 3 of site cb (parity p); columns [colour][channel][spin][re, im]
+__device__ __forceinline__ void store_act(uint32_t acc, int warp, __half2* __restrict__ out, int p, int cb, int Vh) {
+  const int grp = warp >> 2, lane0 = (warp & 3) * 32;
+  __half2* q = out + act_at(p, cb, act_blocks(Vh));
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v[3][16];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) tmem_ld16(acc + ((uint32_t)lane0 << 16) + r * 64 + grp * 32 + h * 16, v[r]);
+    if (cb < Vh) {
+#pragma unroll
+      for (int o = 0; o < 2; ++o)
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+          q[((4 * grp + 2 * h + o) * 12 + k) * kSiteBlock] =
+              __floats2half2_rn(v[k % 3][o * 8 + (k / 3) * 2], v[k % 3][o * 8 + (k / 3) * 2 + 1]);
+    }
   }
 }
 
-// the gather of one stage by one thread: part p of the site's (direction, channel) items.
-// C_in = 8: one direction per stage, channels p and p + 4 (one link, 24 loads in flight);
-// C_in = 1: the four parts take the stage's four directions (the last stage's parts
-// 1 to 3 write the zero padding).
-template <int CIN, int K>
-__device__ __forceinline__ void gather_stage(const Geom& g, const float4* __restrict__ U32,
-                                             const __half2* __restrict__ in, size_t V, bool live, const int x[4],
-                                             int st, int part, unsigned char* A, int row, int a_tile) {
-  if (CIN == 1) {
-    const int di = 4 * st + part;
-    const bool on = live && di < 9;
-    Hop h;
-    cplx<float> v[4][3];
-    if (on) {
-      make_hop(g, U32, x, dir_of(di), h);
-      load_channel<1>(in, V, h.sy, 0, v);
-    }
-    store_channel<K>(h, v, on, A, row, part * 8, a_tile);
-  } else {
-    Hop h;
-    cplx<float> v0[4][3], v1[4][3];
-    const int ic0 = part, ic1 = part + 4;
-    if (live) {
-      make_hop(g, U32, x, dir_of(st), h);
-      load_channel<8>(in, V, h.sy, ic0, v0);
-      load_channel<8>(in, V, h.sy, ic1, v1);
-    }
-    store_channel<K>(h, v0, live, A, row, ic0 * 8, a_tile);
-    store_channel<K>(h, v1, live, A, row, ic1 * 8, a_tile);
-  }
-}
-
-// network input: sigma * (even FP32 field [6][Vh] float4) on even sites, 0 on odd sites,
-// as FP16 complex [12][V] (lexicographic sites)
-// rr (optional): |src|^2 already known to the caller (FGCR's residual norm); sigma is then
-// computed here, stored for the later kernels, and no separate reduction is needed
-__global__ void k_embed16(Geom g, const float4* __restrict__ src, float* __restrict__ sigma_p,
-                          __half2* __restrict__ dst, const int* __restrict__ skip, const double* __restrict__ rr) {
-  if (skip && *skip) return;
-  if (rr) {
-    const double t = *rr;
-    const float sg0 = t > 0 ? (float)sqrt(24.0 * g.Vh / t) : 1.0f;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *sigma_p = sg0;
-  }
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  int r = s, x[4];
-  x[0] = r % g.L[0];
-  r /= g.L[0];
-  x[1] = r % g.L[1];
-  r /= g.L[1];
-  x[2] = r % g.L[2];
-  x[3] = r / g.L[2];
-  const bool even = ((x[0] + x[1] + x[2] + x[3]) & 1) == 0;
-  const float sg = rr ? (*rr > 0 ? (float)sqrt(24.0 * g.Vh / *rr) : 1.0f) : *sigma_p;
-  const int cb = s >> 1;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    float4 v = even ? src[(size_t)k * g.Vh + cb] : make_float4(0.f, 0.f, 0.f, 0.f);
-    dst[(size_t)(2 * k) * g.V + s] = __floats2half2_rn(sg * v.x, sg * v.y);
-    dst[(size_t)(2 * k + 1) * g.V + s] = __floats2half2_rn(sg * v.z, sg * v.w);
-  }
-}
-
-// last layer, second half: out(x) = sum_d U_d(x) z_d(x + d) on even sites (the only ones
-// the network output is read on): z_0(x) + sum_mu [U_mu(x) z_{1+mu}(x + mu)
-// + U_mu(x - mu)^dag z_{5+mu}(x - mu)] with the fermion boundary factor on time hops; z
-// is FP16 [9][12][V] scaled by sigma, out the even FP32 field [6][Vh] divided by sigma
-__global__ void k_last_stencil(Geom g, const float4* __restrict__ U32, const __half2* __restrict__ z,
-                               float4* __restrict__ out, const float* __restrict__ sigma_p,
-                               const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  const int cb = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cb >= g.Vh) return;
-  int x[4];
-  cb_coords(g, cb, 0, x);
-  const size_t V = (size_t)g.V;
-  cplx<float> acc[12];
-  {
-    const size_t s0 = (size_t)lex_index(g, x);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const float2 v = __half22float2(__ldg(z + (size_t)k * V + s0));
-      acc[k] = mk(v.x, v.y);
-    }
-  }
-#pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-      int y[4] = {x[0], x[1], x[2], x[3]};
-      float f = 1.0f;
-      Mat3<float> Um;
-      if (dir == 0) {
-        y[mu] = y[mu] + 1 == g.L[mu] ? 0 : y[mu] + 1;
-        if (mu == 3 && x[3] == g.L[3] - 1) f = (float)g.bc_t;
-        load_link(Um, U32 + (size_t)(mu * 3) * g.Vh, cb, g.Vh);  // x is even: parity 0
-      } else {
-        y[mu] = y[mu] == 0 ? g.L[mu] - 1 : y[mu] - 1;
-        if (mu == 3 && x[3] == 0) f = (float)g.bc_t;
-        Mat3<float> L;
-        load_link(L, U32 + (size_t)((4 + mu) * 3) * g.Vh, cb_index(g, y), g.Vh);  // y is odd
-        Um = dagger(L);
-      }
-      const int d = dir == 0 ? 1 + mu : 5 + mu;
-      const size_t sy = (size_t)lex_index(g, y);
-      cplx<float> v[4][3];
-#pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float2 w = __half22float2(__ldg(z + ((size_t)d * 12 + sp * 3 + c) * V + sy));
-          v[sp][c] = mk(w.x, w.y);
-        }
-#pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-          acc[sp * 3 + r] = acc[sp * 3 + r] + f * (Um.m[r][0] * v[sp][0] + Um.m[r][1] * v[sp][1] + Um.m[r][2] * v[sp][2]);
-    }
-  }
-  const float inv = 1.0f / *sigma_p;
-#pragma unroll
-  for (int j = 0; j < 6; ++j)
-    out[(size_t)j * g.Vh + cb] =
-        make_float4(inv * acc[2 * j].re, inv * acc[2 * j].im, inv * acc[2 * j + 1].re, inv * acc[2 * j + 1].im);
-}
-
-// OUT16: FP16 scaled output for the next layer; otherwise FP32 output divided by sigma
-template <int CIN, int COUT, bool OUT16>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_nn_layer_tc(Geom g, const float4* __restrict__ U32, const __half* __restrict__ Bg, const __half2* __restrict__ in,
-                  void* __restrict__ out, const float* __restrict__ sigma_p, int* __restrict__ err,
-                  const int* __restrict__ skip) {
-  using S = Shape<CIN, COUT>;
+// ---------------------------------------------------------------- one-stage layers
+// Per tile: gather, MMA, epilogue; two resident blocks per SM overlap each other's phases.
+// Thread (row, half).  First layer: even sites, half 0 takes the site's spinor and half 1 the
+// padding slot; odd sites, half h takes the hops of mu = 2 h and 2 h + 1.  The input is rounded
+// to FP16 before the transport.  Last layer: half h copies the channels 4 h .. 4 h + 3; the
+// output z has the layout of the activations, with the hop 1 + o in place of channel o on odd
+// sites and z_0 in place of channel 0 on even ones.
+// rr (first layer, optional): |in|^2 known to the caller (FGCR); sigma then comes from it and
+// is stored for the last layer.
+template <bool FIRST>
+__global__ void __launch_bounds__(kGather, 2)
+    k_nn_single(Geom g, const float4* __restrict__ U32, const __half* __restrict__ Bg, const void* __restrict__ in,
+                __half2* __restrict__ out, float* __restrict__ sigma_p, const double* __restrict__ rr, int* __restrict__ err,
+                const int* __restrict__ skip) {
+  using S = Single<FIRST>;
   if (skip && *skip) return;  // block-uniform: nothing allocated yet
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint32_t tmem_slot;
-  __shared__ __align__(8) uint64_t bar_w, bar_a[2];
+  __shared__ __align__(8) uint64_t bar_w, bar_m;
   unsigned char* sB = sm;
-  unsigned char* sA = sm + S::B_ALL;
-  const int tid = threadIdx.x;
-  const int row = tid & (kM - 1);  // site in the tile
-  const int part = tid >> 7;       // which of the site's (direction, channel) items
-  const size_t V = (size_t)g.V;
-  const float inv_sigma = OUT16 ? 1.0f : 1.0f / *sigma_p;
-
+  unsigned char* A = sm + S::B_ALL;
+  const int tid = threadIdx.x, row = tid & (kM - 1), half = tid >> 7, warp = tid >> 5;
+  const int Vh = g.Vh;
+  const float bcf = (float)g.bc_t;
+  float sigma = 1.f;
+  if (FIRST) {
+    if (rr) {
+      sigma = sigma_of(*rr, Vh);
+      if (blockIdx.x == 0 && tid == 0) *sigma_p = sigma;
+    } else {
+      sigma = *sigma_p;
+    }
+  }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar_w)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar_a[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar_a[1])));
+    mbar_init(&bar_w, 1);
+    mbar_init(&bar_m, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (tid < 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
-                 "r"(S::TMEM_COLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (tid < 32) tmem_alloc(&tmem_slot, S::TMEM_COLS);
+  fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-
-  // weights of all stages: bulk TMA copies completing on bar_w
+  fence_after();
+  const uint32_t tmem = tmem_slot, barw = smem_addr(&bar_w), barm = smem_addr(&bar_m);
   if (tid == 0) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar_w)), "r"(S::B_ALL)
-                 : "memory");
-    for (int st = 0; st < S::NST; ++st)
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-              smem_addr(sB + st * S::B_ST)),
-          "l"(Bg + (size_t)st * (S::B_ST / 2)), "r"(S::B_ST), "r"(smem_addr(&bar_w))
-          : "memory");
+    expect_tx(barw, S::B_ALL);
+    bulk_load(sB, Bg, S::B_ALL, barw);
   }
-  bool fail = !mbar_wait(smem_addr(&bar_w), 0);
+  bool fail = !mbar_wait(barw, 0);
   if (fail) atomicExch(err, 1);
-  // every abort decision below is block-uniform (__syncthreads_or of the threads' own
-  // wait results), so all threads leave the loops together
+  // the abort decisions are block-uniform (__syncthreads_or of the threads' wait results)
   bool aborted = __syncthreads_or(fail);
-
-  const int ntiles = (g.V + kM - 1) / kM;
-  uint32_t use = 0;           // A-buffer uses issued so far (buffer = use & 1)
-  int pending[2] = {-1, -1};  // use index of the last commit on each buffer (thread 0 view)
-  const uint32_t id = idesc(kM, S::N);
-  for (int tile = blockIdx.x; tile < ntiles && !aborted; tile += gridDim.x) {
-    const int s = tile * kM + row;
-    const bool live = s < g.V;
-    int x[4] = {0, 0, 0, 0};
-    if (live) {
-      int r = s;
-      x[0] = r % g.L[0];
-      r /= g.L[0];
-      x[1] = r % g.L[1];
-      r /= g.L[1];
-      x[2] = r % g.L[2];
-      x[3] = r / g.L[2];
-    }
-    for (int st = 0; st < S::NST; ++st, ++use) {
-      const int buf = use & 1;
-      // the MMAs that last read this buffer (use - 2) must be complete
-      fail = use >= 2 && !mbar_wait(smem_addr(&bar_a[buf]), ((use >> 1) - 1) & 1);
-      if (fail) atomicExch(err, 2);
-      unsigned char* A = sA + buf * S::A_BUF;
-      // ---- gather of the stage's inputs into the three colour tiles
-      gather_stage<CIN, S::K>(g, U32, in, V, live, x, st, part, A, row, S::A_TILE);
-      // ---- make the tiles visible to the tensor core, then one thread issues the MMAs
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      if (__syncthreads_or(fail)) {
-        aborted = true;
-        break;
+  const int nt = (Vh + kM - 1) / kM;
+  uint32_t n = 0;        // tiles done: parity of bar_m
+  bool pending = false;  // MMAs committed and not waited for (thread 0)
+  for (int t = blockIdx.x; t < 2 * nt && !aborted; t += gridDim.x, ++n) {
+    const int p = t & 1, cb = (t >> 1) * kM + row;
+    const int cs = cb < Vh ? cb : Vh - 1;  // rows past the end gather a valid site and are not stored
+    if constexpr (!FIRST) {
+      const uint32_t* w = (const uint32_t*)in + act_at(p, cs, act_blocks(Vh)) + half * (48 * kSiteBlock);
+      uint32_t raw[4][12];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 12; ++k) raw[c][k] = __ldg(w + (c * 12 + k) * kSiteBlock);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) store_row(A, S::A_TILE, kmajor(row, (4 * half + c) * 8, S::KD), raw[c]);
+    } else {
+      auto spinor16 = [&](int site, uint32_t w[12]) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const float4 v = __ldg((const float4*)in + (size_t)k * Vh + site);
+          w[2 * k] = pack_h2(sigma * v.x, sigma * v.y);
+          w[2 * k + 1] = pack_h2(sigma * v.z, sigma * v.w);
+        }
+      };
+      uint32_t w[12];
+      if (p == 0 && half == 0) {
+        spinor16(cs, w);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) w[k] = 0;
       }
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // even: slot 0 the site, slot 1 zero; odd: slots 0 and 9 zero
+      store_row(A, S::A_TILE, kmajor(row, (half == 0 ? 0 : (p == 0 ? 1 : 9)) * 8, S::KD), w);
+      if (p == 1) {
+        const Site s = site_at(g, cs, 1);
+        auto hop = [&](auto fwd, int i) {
+          bool edge;
+          const int nb = hop_site(g, s, i, edge);
+          float4 l[3];
+          load_link_raw(l, U32, Vh, 1, i, cs, nb);
+          spinor16(nb, w);
+          const Mat3x2 P = pair_matrix(transport_matrix<decltype(fwd)::value>(l, edge, bcf));
+          transport_pair(P, w, w + 3, w, w + 3);
+          transport_pair(P, w + 6, w + 9, w + 6, w + 9);
+          store_row(A, S::A_TILE, kmajor(row, i * 8, S::KD), w);
+        };
 #pragma unroll 1
-        for (int r = 0; r < 3; ++r) {
-          const uint32_t a0 = smem_addr(A + r * S::A_TILE);
-          const uint32_t b0 = smem_addr(sB + st * S::B_ST);
-#pragma unroll 1
-          for (int kk = 0; kk < S::K / 16; ++kk)
-            mma_f16(tmem + r * S::N, sdesc(a0 + kk * 256, 128, S::SBO), sdesc(b0 + kk * 256, 128, S::SBO), id,
-                    (st > 0 || kk > 0) ? 1u : 0u);
+        for (int i = 4 * half + 1; i < 4 * half + 5; i += 2) {
+          hop(std::true_type(), i);
+          hop(std::false_type(), i + 1);
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_addr(&bar_a[buf]))
-                     : "memory");
-        pending[buf] = (int)use;
-      }
-    }
-    if (aborted) break;
-    // ---- epilogue: all MMAs of the tile are complete when the last commit has arrived
-    const uint32_t last = use - 1;
-    fail = !mbar_wait(smem_addr(&bar_a[last & 1]), (last >> 1) & 1);
-    if (fail) atomicExch(err, 3);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (__syncthreads_or(fail)) {
-      aborted = true;
-      break;
-    }
-    if (tid == 0) pending[0] = pending[1] = -1;
-    {
-      // warp w reads TMEM lanes 32 (w % 4) .. + 31; the 16-column chunks are dealt out
-      // to the four column groups w / 4
-      const int w = tid >> 5, q = w & 3, grp = w >> 2;
-      const int srow = tile * kM + q * 32 + (tid & 31);
-      constexpr int NCHUNK = 3 * S::N / 16;
-#pragma unroll 1
-      for (int chunk = grp; chunk < NCHUNK; chunk += kThreads / 128) {
-        const int c0 = chunk * 16;
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + c0, v);
-        if (srow < g.V) {
-#pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            const int col = c0 + j;
-            const int r = col / S::N, n = col % S::N;
-            const int o = n >> 3, a = (n >> 1) & 3;
-            if (o < COUT) {
-              const size_t idx = ((size_t)o * 12 + a * 3 + r) * V + srow;
-              if (OUT16)
-                reinterpret_cast<__half2*>(out)[idx] = __floats2half2_rn(v[j], v[j + 1]);
-              else
-                reinterpret_cast<float2*>(out)[idx] = make_float2(v[j] * inv_sigma, v[j + 1] * inv_sigma);
-            }
-          }
-        }
-      }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-  }
-  // ---- teardown: nothing of this CTA may still be running on the tensor core
-  if (tid == 0) {
-    for (int b = 0; b < 2; ++b)
-      if (pending[b] >= 0) mbar_wait(smem_addr(&bar_a[b]), ((uint32_t)pending[b] >> 1) & 1);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::TMEM_COLS));
-}
-
-// ---------------------------------------------------------------- pipelined layer (C_out = 8)
-// The same contraction with the gather split in two: the raw neighbour activations go
-// global -> shared by 4-byte cp.async copies (no registers held; the threads of a warp,
-// consecutive sites, copy consecutive words), one stage ahead of the stage being
-// transported; the links of the next stage are prefetched into registers.  Per stage:
-// issue the copies of stage u + 1, wait for those of stage u, transport them from the
-// staging buffer into the FP16 A tiles, one thread issues the MMAs.  Staging layout
-// [slot][component][row] (slot: the input channel, or for C_in = 1 the direction of the
-// stage), so the warp's reads in the transport are conflict-free.  The A tiles are
-// single-buffered: the transport of stage u waits for the MMAs of stage u - 1.
-template <int CIN>
-struct Pipe {
-  using S = Shape<CIN, 8>;
-  static constexpr int SLOTS = CIN == 1 ? 4 : 8;
-  static constexpr int STAGE_BYTES = SLOTS * 12 * kM * 4;
-  static constexpr int SMEM = S::B_ALL + S::A_BUF + 2 * STAGE_BYTES;
-  static_assert(SMEM <= 227 * 1024, "shared memory");
-};
-
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
-
-// the next stage's item of one thread: neighbour site, boundary factor, kind and the raw
-// 12-real link (rebuilt and daggered at transport time)
-struct HopRaw {
-  float4 l[3];
-  float f;
-  int kind;  // 0 site, 1 forward, 2 backward, -1 nothing (padding or a dead row)
-};
-
-__device__ __forceinline__ void hop_prefetch(const Geom& g, const float4* __restrict__ U32, const int x[4], int d,
-                                             HopRaw& h, size_t& sy) {
-  h.kind = d == 0 ? 0 : (d <= 4 ? 1 : 2);
-  const int mu = d == 0 ? 0 : (d - 1) & 3;
-  int y[4] = {x[0], x[1], x[2], x[3]};
-  h.f = 1.0f;
-  if (h.kind == 1) {
-    y[mu] = y[mu] + 1 == g.L[mu] ? 0 : y[mu] + 1;
-    if (mu == 3 && x[3] == g.L[3] - 1) h.f = (float)g.bc_t;
-    const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-    const float4* l = U32 + (size_t)((p * 4 + mu) * 3) * g.Vh + cb_index(g, x);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) h.l[k] = __ldg(l + (size_t)k * g.Vh);
-  } else if (h.kind == 2) {
-    y[mu] = y[mu] == 0 ? g.L[mu] - 1 : y[mu] - 1;
-    if (mu == 3 && x[3] == 0) h.f = (float)g.bc_t;
-    const int p = (y[0] + y[1] + y[2] + y[3]) & 1;
-    const float4* l = U32 + (size_t)((p * 4 + mu) * 3) * g.Vh + cb_index(g, y);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) h.l[k] = __ldg(l + (size_t)k * g.Vh);
-  }
-  sy = (size_t)lex_index(g, y);
-}
-
-__device__ __forceinline__ void site_coords(const Geom& g, int s, int x[4]) {
-  int r = s;
-  x[0] = r % g.L[0];
-  r /= g.L[0];
-  x[1] = r % g.L[1];
-  r /= g.L[1];
-  x[2] = r % g.L[2];
-  x[3] = r / g.L[2];
-}
-
-template <int CIN>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_nn_layer_tc2(Geom g, const float4* __restrict__ U32, const __half* __restrict__ Bg, const __half2* __restrict__ in,
-                   __half2* __restrict__ out, int* __restrict__ err, const int* __restrict__ skip) {
-  using S = Shape<CIN, 8>;
-  using PP = Pipe<CIN>;
-  if (skip && *skip) return;
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ uint32_t tmem_slot;
-  __shared__ __align__(8) uint64_t bar_w, bar_a;
-  unsigned char* sB = sm;
-  unsigned char* sA = sm + S::B_ALL;
-  unsigned char* sR = sm + S::B_ALL + S::A_BUF;  // two staging buffers
-  const int tid = threadIdx.x;
-  const int row = tid & (kM - 1);
-  const int part = tid >> 7;
-
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar_w)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar_a)));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (tid < 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
-                 "r"(S::TMEM_COLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  if (tid == 0) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar_w)), "r"(S::B_ALL)
-                 : "memory");
-    for (int st = 0; st < S::NST; ++st)
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-              smem_addr(sB + st * S::B_ST)),
-          "l"(Bg + (size_t)st * (S::B_ST / 2)), "r"(S::B_ST), "r"(smem_addr(&bar_w))
-          : "memory");
-  }
-  bool fail = !mbar_wait(smem_addr(&bar_w), 0);
-  if (fail) atomicExch(err, 1);
-  bool aborted = __syncthreads_or(fail);
-
-  const int ntiles = (g.V + kM - 1) / kM;
-  const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  const int nwork = my_tiles * S::NST;
-  const uint32_t id = idesc(kM, S::N);
-
-  // issue the copies (and link loads) of work item u into staging buffer u & 1
-  auto issue = [&](int u, HopRaw& h) {
-    h.kind = -1;
-    if (u >= nwork) return;
-    const int tile = blockIdx.x + (u / S::NST) * gridDim.x, st = u % S::NST;
-    const int s = tile * kM + row;
-    if (s >= g.V) return;
-    int x[4];
-    site_coords(g, s, x);
-    const int di = CIN == 1 ? 4 * st + part : st;
-    if (di >= 9) return;
-    size_t sy;
-    hop_prefetch(g, U32, x, dir_of(di), h, sy);
-    const uint32_t base = smem_addr(sR + (u & 1) * PP::STAGE_BYTES) + row * 4;
-    const size_t V = (size_t)g.V;
-    // C_in = 8: channels 2 part, 2 part + 1; C_in = 1: the part's direction slot
-#pragma unroll
-    for (int q = 0; q < (CIN == 1 ? 1 : 2); ++q) {
-      const int ic = CIN == 1 ? 0 : 2 * part + q;
-      const int slot = CIN == 1 ? part : ic;
-#pragma unroll
-      for (int k = 0; k < 12; ++k)
-        cp_async4(base + (uint32_t)((slot * 12 + k) * kM) * 4, in + ((size_t)ic * 12 + k) * V + sy);
-    }
-  };
-
-  HopRaw cur, nxt;
-  if (!aborted) issue(0, cur);
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  uint32_t commits = 0;  // MMA commits issued on bar_a
-  for (int u = 0; u < nwork && !aborted; ++u) {
-    const int tl = u / S::NST, st = u % S::NST;
-    const int tile = blockIdx.x + tl * gridDim.x;
-    issue(u + 1, nxt);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    // the MMAs of the previous stage read the A tiles: wait for them
-    fail = commits > 0 && !mbar_wait(smem_addr(&bar_a), (commits - 1) & 1);
-    if (fail) atomicExch(err, 2);
-    if (__syncthreads_or(fail)) {
-      aborted = true;
-      break;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- transport the staged inputs into the three colour tiles
-    {
-      const uint32_t* R = reinterpret_cast<const uint32_t*>(sR + (u & 1) * PP::STAGE_BYTES) + row;
-      Hop h;
-      h.kind = cur.kind < 0 ? 0 : cur.kind;
-      h.f = cur.f;
-      if (cur.kind > 0) {
-        Mat3<float> L;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          L.m[(2 * k) / 3][(2 * k) % 3] = mk(cur.l[k].x, cur.l[k].y);
-          L.m[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(cur.l[k].z, cur.l[k].w);
-        }
-        reconstruct_row2(L);
-        h.U = cur.kind == 1 ? L : dagger(L);
-      }
-      const bool live = cur.kind >= 0;
-      constexpr int NCH = CIN == 1 ? 1 : 2;
-#pragma unroll
-      for (int q = 0; q < NCH; ++q) {
-        const int slot = CIN == 1 ? part : 2 * part + q;
-        cplx<float> v[4][3];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          const float2 f = live ? h2_to_f2(R[(slot * 12 + k) * kM]) : make_float2(0.f, 0.f);
-          v[k / 3][k % 3] = mk(f.x, f.y);
-        }
-        const int col = CIN == 1 ? part * 8 : (2 * part + q) * 8;
-        store_channel<S::K>(h, v, live, sA, row, col, S::A_TILE);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    fence_before();
     __syncthreads();
     if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
+      fence_after();
+      const uint32_t b0 = smem_addr(sB + (p ? S::B_EVEN : 0));
+      const int K = p ? S::KD : S::K_EVEN;
+      const uint32_t id = idesc(kM, p ? S::N_ODD : S::N_EVEN);
       for (int r = 0; r < 3; ++r) {
-        const uint32_t a0 = smem_addr(sA + r * S::A_TILE);
-        const uint32_t b0 = smem_addr(sB + st * S::B_ST);
-#pragma unroll 1
-        for (int kk = 0; kk < S::K / 16; ++kk)
-          mma_f16(tmem + r * S::N, sdesc(a0 + kk * 256, 128, S::SBO), sdesc(b0 + kk * 256, 128, S::SBO), id,
-                  (st > 0 || kk > 0) ? 1u : 0u);
+        const uint32_t a0 = smem_addr(A + r * S::A_TILE);
+        for (int kk = 0; kk < K / 16; ++kk)
+          mma_f16(tmem + r * 64, sdesc(a0 + kk * 256, 128, 16 * S::KD), sdesc(b0 + kk * 256, 128, 16 * K), id, kk > 0);
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_addr(&bar_a))
-                   : "memory");
+      mma_commit(barm);
+      pending = true;
     }
-    ++commits;
-    cur = nxt;
-    if (st == S::NST - 1) {
-      // ---- epilogue of the tile: accumulators complete when the last commit arrived
-      fail = !mbar_wait(smem_addr(&bar_a), (commits - 1) & 1);
-      if (fail) atomicExch(err, 3);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (__syncthreads_or(fail)) {
-        aborted = true;
-        break;
-      }
-      // warp w: TMEM lanes 32 (w % 4) .. + 31 (sites), output channels 2 (w / 4), + 1;
-      // channel-major output [8][12][V]: consecutive lanes write consecutive sites
-      const int w = tid >> 5, qd = w & 3, grp = w >> 2;
-      const int srow = tile * kM + qd * 32 + (tid & 31);
-      const size_t V = (size_t)g.V;
+    fail = !mbar_wait(barm, n & 1);
+    if (fail) atomicExch(err, 2);
+    aborted = __syncthreads_or(fail);
+    if (aborted) break;
+    pending = false;
+    fence_after();
+    const int c = (t >> 1) * kM + (warp & 3) * 32 + (tid & 31);
+    if (FIRST || p == 1) {
+      store_act(tmem, warp, out, p, c, Vh);
+    } else if (warp < 4) {
       float v[3][16];
 #pragma unroll
-      for (int r = 0; r < 3; ++r) tmem_ld16(tmem + ((uint32_t)(qd * 32) << 16) + r * S::N + grp * 16, v[r]);
-      if (srow < g.V) {
+      for (int r = 0; r < 3; ++r) tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + r * 64, v[r]);
+      if (c < Vh) {
+        __half2* q = out + act_at(0, c, act_blocks(Vh));
 #pragma unroll
-        for (int o = 0; o < 2; ++o)
-#pragma unroll
-          for (int k = 0; k < 12; ++k) {  // complex k = spin a * 3 + colour r
-            const int a = k / 3, r = k % 3;
-            out[((size_t)(2 * grp + o) * 12 + k) * V + srow] =
-                __floats2half2_rn(v[r][o * 8 + a * 2], v[r][o * 8 + a * 2 + 1]);
-          }
+        for (int k = 0; k < 12; ++k) q[k * kSiteBlock] = __floats2half2_rn(v[k % 3][(k / 3) * 2], v[k % 3][(k / 3) * 2 + 1]);
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
+    }
+    fence_before();
+    __syncthreads();
+  }
+  if (tid == 0 && pending) mbar_wait(barm, n & 1);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (tid < 32) tmem_free(tmem, S::TMEM_COLS);
+}
+
+// The network's output on even sites, out(x) = (z_0(x) + sum_d U_d(x) z_d(x + d)) / sigma: a
+// block takes 32 sites, warp mu both hops of direction mu (48 words in flight per thread where
+// one thread per site looped over the hops: 40 us at 16^3x32), the sums meet in shared memory.
+__global__ void __launch_bounds__(128) k_nn_last(Geom g, const float4* __restrict__ U32, const uint32_t* __restrict__ z,
+                                                 float4* __restrict__ out, const float* __restrict__ sigma_p,
+                                                 const int* __restrict__ skip) {
+  if (skip && *skip) return;
+  __shared__ float2 sh[4][12][32];
+  const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
+  const int cb = blockIdx.x * 32 + lane, Vh = g.Vh, cs = cb < Vh ? cb : Vh - 1;
+  const size_t nb32 = act_blocks(Vh);
+  const Site s = site_at(g, cs, 0);
+  const float bcf = (float)g.bc_t;
+  uint32_t w[2][12];
+  float4 l[2][3];
+  bool edge[2];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const int i = 2 * mu + 1 + b;  // stage: +mu, -mu
+    const int nb = hop_site(g, s, i, edge[b]);
+    const uint32_t* q = z + act_at(1, nb, nb32) + (dir_of(i) - 1) * (12 * kSiteBlock);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) w[b][k] = __ldg(q + k * kSiteBlock);
+    load_link_raw(l[b], U32, Vh, 0, i, cs, nb);
+  }
+  cplx<float> acc[12];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const Mat3<float> M = b == 0 ? transport_matrix<true>(l[b], edge[b], bcf) : transport_matrix<false>(l[b], edge[b], bcf);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const int sp = k / 3, r = k % 3;
+      cplx<float> y = b ? acc[k] : mk(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float2 v = h2_to_f2(w[b][3 * sp + c]);
+        y = cmad(M.m[r][c], mk(v.x, v.y), y);
+      }
+      acc[k] = y;
     }
   }
-  // ---- teardown: no copy in flight, nothing of this CTA running on the tensor core
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  if (tid == 0 && commits > 0) mbar_wait(smem_addr(&bar_a), (commits - 1) & 1);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 12; ++k) sh[mu][k][lane] = make_float2(acc[k].re, acc[k].im);
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::TMEM_COLS));
+  const float inv = 1.0f / *sigma_p;
+  for (int j = mu; j < 6; j += 4) {  // components 2 j, 2 j + 1
+    float2 o[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int k = 2 * j + e;
+      o[e] = h2_to_f2(__ldg(z + act_at(0, cs, nb32) + k * kSiteBlock));
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        o[e].x += sh[m][k][lane].x;
+        o[e].y += sh[m][k][lane].y;
+      }
+    }
+    if (cb < Vh) out[(size_t)j * Vh + cb] = make_float4(inv * o[0].x, inv * o[0].y, inv * o[1].x, inv * o[1].y);
+  }
+}
+
+// ---------------------------------------------------------------- hidden layer
+// Warps 0-7 gather and transport (thread (row, half): channels 4 half .. 4 half + 3), warp 8
+// issues the MMAs.  Per stage: wait until the A buffer is free (MMAs of two stages before),
+// transport the prefetched words into it and refill their registers for the next stage (the
+// next tile's first stage after the ninth), arrive on full.  Rows past the end of the lattice
+// gather the last site and are not stored.
+__global__ void __launch_bounds__(kGather + 32, 1)
+    k_nn_hidden(Geom g, const float4* __restrict__ U32, const __half* __restrict__ Bg, const uint32_t* __restrict__ in,
+                __half2* __restrict__ out, int* __restrict__ err, const int* __restrict__ skip) {
+  using S = Hidden;
+  if (skip && *skip) return;  // block-uniform: nothing allocated yet
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint32_t tmem_slot;
+  __shared__ __align__(8) uint64_t bar_w, bar_full[2], bar_free[2], bar_acc[2], bar_read[2];
+  unsigned char* sB = sm;
+  unsigned char* sA = sm + S::B_ALL;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int Vh = g.Vh;
+  if (tid == 0) {
+    mbar_init(&bar_w, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&bar_full[b], kGather / 32);
+      mbar_init(&bar_free[b], 1);
+      mbar_init(&bar_acc[b], 1);
+      mbar_init(&bar_read[b], kGather / 32);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (tid < 32) tmem_alloc(&tmem_slot, S::TMEM_COLS);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tmem_slot;
+  const int ntiles = 2 * ((Vh + kM - 1) / kM);  // parity t & 1
+
+  if (warp == kGather / 32) {
+    // ---- MMA issue: one thread
+    if ((tid & 31) == 0) {
+      const uint32_t barw = smem_addr(&bar_w);
+      expect_tx(barw, S::B_ALL);
+      for (int st = 0; st < S::NST; ++st)
+        bulk_load(sB + st * S::B_ST, Bg + (size_t)st * (S::B_ST / 2), S::B_ST, barw);
+      bool ok = mbar_wait(barw, 0);
+      const uint32_t id = idesc(kM, S::N);
+      uint32_t use = 0, i = 0;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+        const uint32_t set = i & 1;
+        if (i >= 2) ok = mbar_wait(smem_addr(&bar_read[set]), ((i >> 1) - 1) & 1);
+        for (int st = 0; st < S::NST && ok; ++st) {
+          const uint32_t buf = use & 1;
+          ok = mbar_wait(smem_addr(&bar_full[buf]), (use >> 1) & 1);
+          if (!ok) break;
+          fence_after();
+          const uint32_t b0 = smem_addr(sB + st * S::B_ST);
+#pragma unroll 1
+          for (int r = 0; r < 3; ++r) {
+            const uint32_t a0 = smem_addr(sA + buf * kABuf + r * kATile);
+#pragma unroll
+            for (int kk = 0; kk < kK / 16; ++kk)
+              mma_f16(tmem + set * S::SET + r * S::N, sdesc(a0 + kk * 256, 128, 16 * kK), sdesc(b0 + kk * 256, 128, 16 * kK),
+                      id, (st > 0 || kk > 0) ? 1u : 0u);
+          }
+          mma_commit(smem_addr(&bar_free[buf]));
+          ++use;
+        }
+        if (ok) mma_commit(smem_addr(&bar_acc[set]));
+      }
+      if (!ok) atomicExch(err, 2);
+      // nothing may still be running on the tensor core when its memory is freed
+      for (uint32_t b = 0; b < 2; ++b)
+        if (use > b) mbar_wait(smem_addr(&bar_free[(use - 1 - b) & 1]), ((use - 1 - b) >> 1) & 1);
+    }
+  } else {
+    // ---- gather and transport
+    const int row = tid & (kM - 1), half = tid >> 7;
+    const size_t nb32 = act_blocks(Vh);
+    const float bcf = (float)g.bc_t;
+    uint32_t raw[4][12];
+    float4 link[3];
+    bool edge = false, ok = true;
+    int tile = blockIdx.x;
+    Site s{};
+    int p = 0, cb = 0;
+    auto place = [&](int t) {  // the row's site in tile t
+      p = t & 1;
+      const int c = (t >> 1) * kM + row;
+      cb = c < Vh ? c : Vh - 1;
+      s = site_at(g, cb, p);
+    };
+    auto words = [&](int q, int c) {  // activations of this half's channels at site c of parity q
+      return in + act_at(q, c, nb32) + half * (48 * kSiteBlock);
+    };
+    // accumulators of this block's tile number i (tile index t) -> output
+    auto epilogue = [&](uint32_t i, int t) {
+      const uint32_t set = i & 1;
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&bar_acc[set]), (i >> 1) & 1));
+      if (!ok) return;
+      fence_after();
+      store_act(tmem + set * S::SET, warp, out, t & 1, (t >> 1) * kM + (warp & 3) * 32 + (tid & 31), Vh);
+      fence_before();
+      __syncwarp();
+      if ((tid & 31) == 0) mbar_arrive(smem_addr(&bar_read[set]));
+    };
+    if (tile < ntiles) {
+      place(tile);
+      const uint32_t* w = words(p, cb);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 12; ++k) raw[c][k] = __ldg(w + (c * 12 + k) * kSiteBlock);
+    }
+    uint32_t use = 0, i = 0;
+    // stage st of the tile; KIND: 0 the site itself, 1 a forward hop, 2 a backward hop
+    auto stage = [&](auto kind, int st) {
+      constexpr int KIND = decltype(kind)::value;
+      const uint32_t buf = use & 1;
+      if (use >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&bar_free[buf]), ((use >> 1) - 1) & 1));
+      if (!ok) return;
+      Mat3x2 P;
+      if constexpr (KIND != 0) P = pair_matrix(transport_matrix<KIND == 1>(link, edge, bcf));
+      // where the next stage reads: the next hop of this site, or the next tile's own site
+      int nx = cb, np = p;
+      if (KIND != 2 || st + 1 < S::NST) {
+        nx = hop_site(g, s, st + 1, edge);
+        np = 1 - p;
+        load_link_raw(link, U32, Vh, p, st + 1, cb, nx);
+      } else if (tile + (int)gridDim.x < ntiles) {
+        place(tile + gridDim.x);
+        nx = cb;
+        np = p;
+      }
+      const uint32_t* w = words(np, nx);
+      unsigned char* A = sA + buf * kABuf;
+#pragma unroll
+      for (int c = 0; c < 4; c += 2) {
+        if constexpr (KIND != 0) {
+#pragma unroll
+          for (int sp = 0; sp < 4; ++sp) transport_pair(P, &raw[c][3 * sp], &raw[c + 1][3 * sp], &raw[c][3 * sp], &raw[c + 1][3 * sp]);
+        }
+#pragma unroll
+        for (int q = c; q < c + 2; ++q) store_row(A, kATile, kmajor(row, (4 * half + q) * 8, kK), raw[q]);
+#pragma unroll
+        for (int q = c; q < c + 2; ++q)
+#pragma unroll
+          for (int k = 0; k < 12; ++k) raw[q][k] = __ldg(w + (q * 12 + k) * kSiteBlock);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if ((tid & 31) == 0) mbar_arrive(smem_addr(&bar_full[buf]));
+      ++use;
+    };
+    for (; tile < ntiles && ok; tile += gridDim.x, ++i) {
+      stage(std::integral_constant<int, 0>(), 0);
+#pragma unroll 1
+      for (int st = 1; st < S::NST && ok; st += 2) {
+        stage(std::integral_constant<int, 1>(), st);
+        if (st == 1 && ok && i > 0) epilogue(i - 1, tile - gridDim.x);
+        if (ok) stage(std::integral_constant<int, 2>(), st + 1);
+      }
+    }
+    if (ok && i > 0) epilogue(i - 1, tile - gridDim.x);
+    if (!ok && (tid & 31) == 0) atomicExch(err, 3);
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (tid < 32) tmem_free(tmem, S::TMEM_COLS);
 }
 
 }  // namespace tc
 
 // ---------------------------------------------------------------- host side
-// layers with (C_in, C_out) in {(1, 8), (8, 8), (8, 1)} run on the tensor cores
+// networks 1 -> 8 -> ... -> 8 -> 1: layers (1, 8), (8, 8), (8, 1)
 bool nn_tc_supported(int cin, int cout) {
   return (cin == 1 && cout == 8) || (cin == 8 && cout == 8) || (cin == 8 && cout == 1);
 }
 
-// the last layer (8 -> 1) is packed for the local mixing (Shape<8, 9>)
 size_t nn_tc_packed_bytes(int cin, int cout) {
-  if (cin == 1) return tc::Shape<1, 8>::B_ALL;
-  if (cout == 1) return tc::Shape<8, 9>::B_ALL;
-  return tc::Shape<8, 8>::B_ALL;
+  if (cin == 1) return tc::Single<true>::B_ALL;
+  return cout == 1 ? tc::Single<false>::B_ALL : tc::Hidden::B_ALL;
 }
 
-template <int CIN, int COUT>
-static void pack_t(pfmp_ctx* c, const void* W, void* Bp) {
-  using S = tc::Shape<CIN, COUT>;
-  const int n = S::NST * S::N * S::K;
-  tc::k_pack_b<CIN, COUT><<<nblocks(n, 256), 256, 0, c->stream>>>((const float2*)W, (__half*)Bp);
-  PFMP_CHECK_LAUNCH();
-}
+// activations of 8 channels between two layers
+size_t nn_tc_act_bytes(const Geom& g) { return 2 * tc::act_blocks(g.Vh) * tc::kWords * tc::kSiteBlock * 4; }
 
 void nn_tc_pack(pfmp_ctx* c, int cin, int cout, const void* W, void* Bp) {
+  const float2* w = (const float2*)W;
+  __half* B = (__half*)Bp;
   if (cin == 1)
-    pack_t<1, 8>(c, W, Bp);
+    tc::k_pack_single<true><<<nblocks(tc::Single<true>::B_ALL / 2), kBlock, 0, c->stream>>>(w, B);
   else if (cout == 1)
-    pack_t<8, 9>(c, W, Bp);
+    tc::k_pack_single<false><<<nblocks(tc::Single<false>::B_ALL / 2), kBlock, 0, c->stream>>>(w, B);
   else
-    pack_t<8, 8>(c, W, Bp);
+    tc::k_pack_hidden<<<nblocks(tc::Hidden::B_ALL / 2), kBlock, 0, c->stream>>>(w, B);
+  PFMP_CHECK_LAUNCH();
 }
 
 void nn_tc_scale(pfmp_ctx* c, const void* in_even_f32, float* sigma_dev, const int* skip) {
@@ -820,107 +817,46 @@ void nn_tc_scale(pfmp_ctx* c, const void* in_even_f32, float* sigma_dev, const i
   PFMP_CHECK_LAUNCH();
 }
 
-template <int CIN, int COUT, bool OUT16>
-static int layer_init() {
-  using S = tc::Shape<CIN, COUT>;
-  static int sms = 0;
-  if (!sms) {
-    PFMP_CUDA(cudaFuncSetAttribute(tc::k_nn_layer_tc<CIN, COUT, OUT16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   S::SMEM));
-    int dev = 0;
+// kernel attributes set outside any stream capture; returns the number of SMs
+int nn_tc_init() {
+  static const int sms = [] {
+    auto smem = [](auto* k, int bytes) {
+      PFMP_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    };
+    smem(tc::k_nn_single<true>, tc::Single<true>::SMEM);
+    smem(tc::k_nn_single<false>, tc::Single<false>::SMEM);
+    smem(tc::k_nn_hidden, tc::Hidden::SMEM);
+    int dev = 0, n = 0;
     PFMP_CUDA(cudaGetDevice(&dev));
-    PFMP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
+    PFMP_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  }();
   return sms;
 }
 
-template <int CIN>
-static int layer2_init() {
-  static int sms = 0;
-  if (!sms) {
-    PFMP_CUDA(cudaFuncSetAttribute(tc::k_nn_layer_tc2<CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   tc::Pipe<CIN>::SMEM));
-    int dev = 0;
-    PFMP_CUDA(cudaGetDevice(&dev));
-    PFMP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return sms;
-}
+static int parity_tiles(const pfmp_ctx* c) { return 2 * nblocks(c->g.Vh, tc::kM); }
 
-// kernel attributes set outside any stream capture
-void nn_tc_init() {
-  layer_init<1, 8, true>();
-  layer_init<8, 8, true>();
-  layer_init<8, 9, true>();
-  layer2_init<1>();
-  layer2_init<8>();
-}
-
-// The staged variant (k_nn_layer_tc2) measured slower than the single-stage kernel at
-// 16^3 x 32 (one network application 0.77 vs 0.57 ms): with one stage of lookahead it holds
-// about the same bytes in flight per SM (one stage, ~48 KB) and adds a barrier and a
-// shared-memory round trip per stage.  It is kept selectable (PFMP_NN_TC_PIPE=1 in the
-// environment) for profiling; the single-stage kernel is the default.
-static bool use_pipe() {
-  static int v = -1;
-  if (v < 0) {
-    const char* e = std::getenv("PFMP_NN_TC_PIPE");
-    v = (e && e[0] == '1') ? 1 : 0;
-  }
-  return v == 1;
-}
-
-template <int CIN>
-static void layer2_t(pfmp_ctx* c, const void* Bp, const void* in, void* out, int* err, const int* skip) {
-  const int sms = layer2_init<CIN>();
-  const int ntiles = (c->g.V + tc::kM - 1) / tc::kM;
-  const int grid = ntiles < sms ? ntiles : sms;
-  tc::k_nn_layer_tc2<CIN><<<grid, tc::kThreads, tc::Pipe<CIN>::SMEM, c->stream>>>(
-      c->g, c->U32, (const __half*)Bp, (const __half2*)in, (__half2*)out, err, skip);
+// in (even FP32) -> FP16 activations; sigma is read, or with rr (|in|^2) set
+void nn_tc_first(pfmp_ctx* c, const void* Bp, const void* in, void* act, float* sigma, const double* rr, int* err,
+                 const int* skip) {
+  const int grid = std::min(parity_tiles(c), 2 * nn_tc_init());
+  tc::k_nn_single<true><<<grid, tc::kGather, tc::Single<true>::SMEM, c->stream>>>(
+      c->g, c->U32, (const __half*)Bp, in, (__half2*)act, sigma, rr, err, skip);
   PFMP_CHECK_LAUNCH();
 }
-
-template <int CIN, int COUT, bool OUT16>
-static void layer_t(pfmp_ctx* c, const void* Bp, const void* in, void* out, const float* sigma, int* err,
-                    const int* skip) {
-  using S = tc::Shape<CIN, COUT>;
-  const int sms = layer_init<CIN, COUT, OUT16>();
-  const int ntiles = (c->g.V + tc::kM - 1) / tc::kM;
-  const int grid = ntiles < sms ? ntiles : sms;
-  tc::k_nn_layer_tc<CIN, COUT, OUT16><<<grid, tc::kThreads, S::SMEM, c->stream>>>(
-      c->g, c->U32, (const __half*)Bp, (const __half2*)in, out, sigma, err, skip);
+void nn_tc_hidden(pfmp_ctx* c, const void* Bp, const void* in, void* out, int* err, const int* skip) {
+  const int grid = std::min(parity_tiles(c), nn_tc_init());
+  tc::k_nn_hidden<<<grid, tc::kGather + 32, tc::Hidden::SMEM, c->stream>>>(c->g, c->U32, (const __half*)Bp,
+                                                                           (const uint32_t*)in, (__half2*)out, err, skip);
   PFMP_CHECK_LAUNCH();
 }
-
-// in: FP16 scaled activations; out: FP16 scaled (last = false) or FP32 / sigma (last)
-void nn_tc_layer(pfmp_ctx* c, int cin, int cout, bool last, const void* Bp, const void* in, void* out,
-                 const float* sigma, int* err, const int* skip) {
-  PFMP_REQUIRE(!last && cout == 8, PFMP_E_INVALID, "tensor-core layer sequence (the last layer: nn_tc_last)");
-  if (use_pipe()) {
-    if (cin == 1)
-      layer2_t<1>(c, Bp, in, out, err, skip);
-    else
-      layer2_t<8>(c, Bp, in, out, err, skip);
-  } else if (cin == 1) {
-    layer_t<1, 8, true>(c, Bp, in, out, sigma, err, skip);
-  } else {
-    layer_t<8, 8, true>(c, Bp, in, out, sigma, err, skip);
-  }
-}
-
-// the last layer (8 -> 1) as local mixing on the tensor cores (z, FP16 [9][12][V]) and
-// the even-site transport stencil, straight into the even FP32 output field
-void nn_tc_last(pfmp_ctx* c, const void* Bp, const void* in, void* z16, void* out_even_f32, const float* sigma,
-                int* err, const int* skip) {
-  layer_t<8, 9, true>(c, Bp, in, z16, sigma, err, skip);
-  tc::k_last_stencil<<<nblocks(c->g.Vh, 128), 128, 0, c->stream>>>(c->g, c->U32, (const __half2*)z16,
-                                                                   (float4*)out_even_f32, sigma, skip);
+// FP16 activations -> out (even FP32), divided by sigma; z: room for one set of activations
+void nn_tc_last(pfmp_ctx* c, const void* Bp, const void* in, void* z, void* out, float* sigma, int* err, const int* skip) {
+  const int grid = std::min(parity_tiles(c), 2 * nn_tc_init());
+  tc::k_nn_single<false><<<grid, tc::kGather, tc::Single<false>::SMEM, c->stream>>>(
+      c->g, c->U32, (const __half*)Bp, in, (__half2*)z, sigma, nullptr, err, skip);
   PFMP_CHECK_LAUNCH();
-}
-
-void nn_tc_embed(pfmp_ctx* c, const void* in_even_f32, float* sigma, void* act16, const int* skip, const double* rr) {
-  tc::k_embed16<<<nblocks(c->g.V, 256), 256, 0, c->stream>>>(c->g, (const float4*)in_even_f32, sigma,
-                                                             (__half2*)act16, skip, rr);
+  tc::k_nn_last<<<nblocks(c->g.Vh, 32), 128, 0, c->stream>>>(c->g, c->U32, (const uint32_t*)z, (float4*)out, sigma, skip);
   PFMP_CHECK_LAUNCH();
 }
 
