@@ -137,6 +137,7 @@ void hop(pfmp_op* op, int prec, void* out, const void* in, int out_parity, bool 
 void clover_mul(pfmp_op* op, int prec, void* out, const void* in, int parity);
 // out = M-hat in (or dagger); if pAp != nullptr the finisher of the second kernel
 // stores ||out||^2 into *pAp (device scalar) and, when scal != nullptr, alpha = rr/pAp
+void mhat_with_temp(pfmp_op* op, int prec, void* out, const void* in, bool dagger, void* temp);
 void mhat(pfmp_op* op, int prec, void* out, const void* in, bool dagger, double* norm_out,
           CGScalars* scal);
 void kop(pfmp_op* op, int prec, void* out, const void* in, double* pKp_dev, CGScalars* scal);

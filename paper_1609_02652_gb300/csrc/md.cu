@@ -228,21 +228,35 @@ void multishift(pfmp_action* A, pfmp_op* op, const std::vector<cd>& sig, const v
   PFMP_REQUIRE(st == PFMP_OK, st, "multi-shift CG inside the action did not converge");
 }
 
-// half-lattice scratch field i of the force batches in precision prec
-void* fscratch(pfmp_action* A, int prec, int i) {
+// half-lattice scratch field i of the fermion forces in precision prec, kept by the action
+void*& fslot(pfmp_action* A, int prec, int i) {
   auto& v = A->fbuf[prec == PFMP_F64 ? 0 : 1];
-  while ((int)v.size() <= i) v.push_back(dev_alloc(spinor_bytes(A->ctx->g, prec)));
+  if ((int)v.size() <= i) v.resize(i + 1, nullptr);
   return v[i];
 }
+void* fscratch(pfmp_action* A, int prec, int i) {
+  void*& p = fslot(A, prec, i);
+  if (!p) p = dev_alloc(spinor_bytes(A->ctx->g, prec));
+  return p;
+}
+
+// An even field v and what the contractions need of it, all of them on the way to K v:
+//   y = A_oo^{-1} H_oe v,  m = M-hat v,  w = A_oo^{-1} H^dag_oe m,  K v = A_ee m - kappa^2 H^dag_eo w
+struct Images {
+  const void* v;
+  void *y, *m, *w;
+};
 
 // The fermion-force contractions of one precision, collected and summed into F and Hc
 // by one launch of each force kernel per kMaxDerivSets of them (App. C: every force is
-// a sum of Re a^dag dM-hat b over the terms' fields).  The fields handed to add_mhat and
-// add_K are read when the batch is flushed: they must stay unchanged until then, which a
-// ring of kRing fields per caller guarantees (add_K flushes before it would overflow, so
-// at most kMaxDerivSets / 2 K contractions are pending).
+// a sum of Re a^dag dM-hat b over the terms' fields).  The fields of a contraction are
+// read when the batch is flushed, which happens as soon as no further pair would fit: at
+// most kMaxDerivSets - 2 contractions are pending while a caller computes the next fields,
+// so fields taken from a ring of kRing slots stay unchanged long enough, one slot of
+// them being written ahead of its use.
 struct ForceBatch {
   static constexpr int kRing = kMaxDerivSets / 2 + 1;
+  static constexpr int kChain = 8 * kRing;  // scratch index of the chains' fields
   pfmp_action* A;
   int prec;
   DerivBatch b;
@@ -250,41 +264,48 @@ struct ForceBatch {
   // callers flush before they read F or Hc; a batch dropped by an exception is lost
   // with the force it belonged to
   void flush() {
-    deriv_mhat_batch(A->ctx, prec, A->F, A->Hc, b);
+    if (b.n) deriv_mhat_batch(A->ctx, prec, A->F, A->Hc, b);
     b.n = 0;
   }
-  // ring field j of this batch's precision (callers' chains of pending fields)
-  void* ring(int j) { return fscratch(A, prec, 3 * kMaxDerivSets + j % kRing); }
-  // Re a^dag dM-hat b (coef) for the operator op; a, b even fields
-  void add_mhat(pfmp_op* op, const void* a, const void* bf, double coef) {
-    if (b.n == kMaxDerivSets) flush();
-    const int k = b.n;
-    void* y = fscratch(A, prec, kMaxDerivSets + 2 * k);
-    void* w = fscratch(A, prec, kMaxDerivSets + 2 * k + 1);
-    hop_clov_odd(op, prec, y, bf, false);
-    hop_clov_odd(op, prec, w, a, true);
-    const double k2 = op->kappa * op->kappa, kc = op->kappa * op->csw;
-    b.s[k] = DerivSet{a, bf, y, w, -k2 * coef, -kc * coef, k2 * (-kc) * coef};
-    b.n++;
+  void* field(int i) { return fscratch(A, prec, i); }
+  // field v of ring slot j (side 0 or 1: a pair's two fields), and room for its images
+  void* ring(int j, int side = 0) { return field((2 * (j % kRing) + side) * 4); }
+  Images ring_images(const void* v, int j, int side = 0) {
+    const int i = (2 * (j % kRing) + side) * 4;
+    return Images{v, field(i + 1), field(i + 2), field(i + 3)};
   }
-  // Re eta^dag dK chi (coef) for K = M-hat^dag M-hat of op:
-  //   Re (M-hat chi)^dag dM-hat eta + Re (M-hat eta)^dag dM-hat chi
-  // (one contraction with twice the coefficient when eta and chi are the same field)
-  void add_K(pfmp_op* op, const void* eta, const void* chi, double coef) {
-    const int need = eta == chi ? 1 : 2;
-    if (b.n + need > kMaxDerivSets) flush();
-    void* Mchi = fscratch(A, prec, b.n);
-    mhat(op, prec, Mchi, chi, false, nullptr, nullptr);
-    if (eta == chi) {
-      add_mhat(op, Mchi, eta, 2.0 * coef);
-      return;
-    }
-    void* Meta = fscratch(A, prec, b.n + 1);
-    mhat(op, prec, Meta, eta, false, nullptr, nullptr);
-    add_mhat(op, Mchi, eta, coef);
-    add_mhat(op, Meta, chi, coef);
+  // Re a^dag dM-hat b (coef), y and w the odd fields of b and a
+  void add(pfmp_op* op, const void* a, const void* bf, const void* y, const void* w, double coef) {
+    const double k2 = op->kappa * op->kappa, kc = op->kappa * op->csw;
+    b.s[b.n++] = DerivSet{a, bf, y, w, -k2 * coef, -kc * coef, k2 * (-kc) * coef};
+  }
+  void flush_if_full() {
+    if (b.n + 2 > kMaxDerivSets) flush();
+  }
+  // Re v^dag dK u (coef) for K = M-hat^dag M-hat of op:
+  //   Re (M-hat u)^dag dM-hat v + Re (M-hat v)^dag dM-hat u
+  void add_K(pfmp_op* op, const Images& V, const Images& U, double coef) {
+    add(op, U.m, V.v, V.y, U.w, coef);
+    add(op, V.m, U.v, U.y, V.w, coef);
+    flush_if_full();
+  }
+  // the same for u = v: one contraction with twice the coefficient
+  void add_K(pfmp_op* op, const Images& V, double coef) {
+    add(op, V.m, V.v, V.y, V.w, 2.0 * coef);
+    flush_if_full();
   }
 };
+
+// the images of v without K v (three hops), and with it (four, next = K v)
+void images(pfmp_op* op, int prec, const Images& V) {
+  mhat_with_temp(op, prec, V.m, V.v, false, V.y);
+  hop_clov_odd(op, prec, V.w, V.m, true);
+}
+void kop_images(pfmp_op* op, int prec, void* next, const Images& V) {
+  op->kapply += 1;
+  mhat_with_temp(op, prec, V.m, V.v, false, V.y);
+  mhat_with_temp(op, prec, next, V.m, true, V.w);
+}
 
 // clover terms of every operator after the gauge field changed; FP32 field strength
 // (fprec = PFMP_F32) for the link updates inside an MD with FP32 forces
@@ -558,66 +579,146 @@ void action_eval(pfmp_action* A, double* S) {
   for (int i = 0; i < (int)A->t.size(); ++i) S[i] = action_term(A, i);
 }
 
-// The fermion forces with FP32 arithmetic (force_prec = PFMP_F32): the spinor products,
+// The force of a filter term phi^dag Q(K) phi, Q = c prod_k (K - q_k):
+//   dS = Re sum_k eta_k^dag dK chi_k,  chi_{m-1} = c phi, chi_{k-1} = (K - q_k) chi_k,
+//                                      eta_0 = phi, eta_{k+1} = (K - q_k^*) eta_k.
+// Every field that a contraction takes is a step of the chains' own K applications (Images): 8
+// stencils per root, where the contractions' own M-hat applications made it 16.  (Q = c R^dag R
+// with a root of each conjugate pair in R would halve that again, with chains that start
+// from each other; its FP32 force is up to 1.9 times further from the FP64 one at order 64.)
+// MD at 24^3x48 with filters of order 12 and 64, this and the correction force below: 825 ->
+// 600 ms, a 4^4 trajectory 43 -> 38 ms.  The images of chi_k are kept (four half-lattice fields per root) while that takes at most half
+// of the free device memory, and recomputed when eta_k is there otherwise (three stencils
+// more).
+static void force_filter(pfmp_action* A, Term& T, pfmp_op* W, int prec, const void* phi) {
+  pfmp_ctx* c = A->ctx;
+  const int m = (int)T.q.size();
+  ForceBatch fb(A, prec);
+  const int base = ForceBatch::kChain;
+  bool keep = fslot(A, prec, base + 4 * m - 1) != nullptr;
+  if (!keep) {
+    size_t free_b = 0, total_b = 0;
+    PFMP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    keep = 4.0 * m * spinor_bytes(c->g, prec) <= 0.5 * (double)free_b;
+  }
+  // chi_k, and with `keep` its images
+  auto chi = [&](int k) { return fb.field(base + (keep ? 4 * k : k)); };
+  auto kept = [&](int k) {
+    const int i = base + 4 * k;
+    return Images{chi(k), fb.field(i + 1), fb.field(i + 2), fb.field(i + 3)};
+  };
+  caxpby(c, prec, T.c, phi, 0.0, chi(m - 1));
+  for (int k = m - 1; k >= 0; --k) {
+    if (k == 0) {
+      if (keep) images(W, prec, kept(k));
+      break;
+    }
+    if (keep)
+      kop_images(W, prec, chi(k - 1), kept(k));
+    else
+      kop(W, prec, chi(k - 1), chi(k), nullptr, nullptr);
+    caxpby(c, prec, -T.q[k], chi(k), 1.0, chi(k - 1));
+  }
+  for (int k = 0; k < m; ++k) {
+    const Images eta = fb.ring_images(k == 0 ? phi : fb.ring(k), k);
+    if (k + 1 < m) {
+      void* next = fb.ring(k + 1);
+      kop_images(W, prec, next, eta);
+      caxpby(c, prec, -std::conj(T.q[k]), eta.v, 1.0, next);
+    } else {
+      images(W, prec, eta);
+    }
+    Images x;
+    if (keep) {
+      x = kept(k);
+    } else {
+      x = fb.ring_images(chi(k), k, 1);
+      images(W, prec, x);
+    }
+    fb.add_K(W, eta, x, 1.0);
+  }
+  fb.flush();
+}
+
+// The force of a correction term from the solutions x_k = (J - z_k)^{-1} phi.  The poles come
+// in conjugate pairs with conjugate residues, whose contractions are the same two numbers:
+// each pair is taken once with twice the coefficient (and x_k's images once).
+static void force_filtercorr(pfmp_action* A, Term& T, pfmp_op* W, int prec, const std::vector<const void*>& x) {
+  ForceBatch fb(A, prec);
+  for (int k = 0, slot = 0; k < (int)x.size(); ++k) {
+    const int j = T.conj_of[k];
+    if (j < k) continue;  // taken with its conjugate
+    const Images V = fb.ring_images(x[j], slot);
+    images(W, prec, V);
+    if (j == k) {
+      fb.add_K(W, V, -T.r[k].real());
+    } else {
+      void* chib = fb.ring(slot, 1);
+      caxpby(A->ctx, prec, T.r[k], x[k], 0.0, chib);
+      const Images U = fb.ring_images(chib, slot, 1);
+      images(W, prec, U);
+      fb.add_K(W, V, U, -2.0);
+    }
+    ++slot;
+  }
+  fb.flush();
+}
+
+// the ratio term phi^dag W J_b^{-1} W^dag phi, chi = J_b^{-1} W^dag phi:
+//   dS = 2 Re phi^dag dW chi - Re chi^dag dJ_b chi
+static void force_ratio(pfmp_action* A, pfmp_op* W, pfmp_op* Mb, int prec, const void* phi, const void* chi) {
+  ForceBatch fb(A, prec);
+  void *y = fb.ring(1), *w = fb.ring(2);
+  hop_clov_odd(W, prec, y, chi, false);
+  hop_clov_odd(W, prec, w, phi, true);
+  fb.add(W, phi, chi, y, w, 2.0);
+  const Images V = fb.ring_images(chi, 0);
+  images(Mb, prec, V);
+  fb.add_K(Mb, V, -1.0);
+  fb.flush();
+}
+static void force_inv(pfmp_action* A, pfmp_op* W, int prec, const void* chi) {
+  ForceBatch fb(A, prec);
+  const Images V = fb.ring_images(chi, 0);
+  images(W, prec, V);
+  fb.add_K(W, V, -1.0);
+  fb.flush();
+}
+
+// The fermion force of term T.  FP32 arithmetic (force_prec = PFMP_F32): the spinor products,
 // the K chains of the filter force and the multi-shift solve of the correction force in
 // FP32 (solves at the MD tolerance), the CG of the ratio and inverse terms mixed, every
 // contraction summed into the FP64 force.  The MD only needs each force to be a fixed
 // function of the gauge field (then every momentum update is a shear of phase space and
 // the MD map stays reversible and area-preserving), so the trajectory is still exact;
 // the actions at its ends are evaluated as before.
-static void force_f32(pfmp_action* A, Term& T, pfmp_op* W, const void* phi) {
+static void fermion_force(pfmp_action* A, Term& T, pfmp_op* W, const void* phi) {
   pfmp_ctx* c = A->ctx;
-  const size_t b32 = spinor_bytes(c->g, PFMP_F32);
-  float4* phi32 = E32(A, 0);
-  blas_copy(c, phi32, PFMP_F32, phi, PFMP_F64);
+  const int prec = f32_forces(A) ? PFMP_F32 : PFMP_F64;
+  const bool f32 = prec == PFMP_F32;
+  const double tol = f32 ? md_tol(A) : A->def.tol;
+  // a field in the forces' precision: itself, or its FP32 copy i
+  auto in_prec = [&](const void* v, int i) -> const void* {
+    if (!f32) return v;
+    blas_copy(c, E32(A, i), PFMP_F32, v, PFMP_F64);
+    return E32(A, i);
+  };
   if (T.d.kind == PFMP_KIND_FILTER) {
-    const int m = (int)T.q.size();
-    while ((int)A->xs32.size() < m) A->xs32.push_back((float4*)dev_alloc(b32));
-    // chi_{m-1} = c phi, chi_k = (J - q_{k+1}) chi_{k+1}
-    caxpby(c, PFMP_F32, T.c, phi32, 0.0, A->xs32[m - 1]);
-    for (int k = m - 2; k >= 0; --k) {
-      kop(W, PFMP_F32, A->xs32[k], A->xs32[k + 1], nullptr, nullptr);
-      caxpby(c, PFMP_F32, -T.q[k + 1], A->xs32[k + 1], 1.0, A->xs32[k]);
-    }
-    // eta_0 = phi, eta_k = (J - q_{k-1}^*) eta_{k-1}, each in its own ring field
-    ForceBatch fb(A, PFMP_F32);
-    const void* eta = phi32;
-    for (int k = 0; k < m; ++k) {
-      if (k > 0) {
-        void* next = fb.ring(k);
-        kop(W, PFMP_F32, next, eta, nullptr, nullptr);
-        caxpby(c, PFMP_F32, -std::conj(T.q[k - 1]), eta, 1.0, next);
-        eta = next;
-      }
-      fb.add_K(W, eta, A->xs32[k], 1.0);
-    }
-    fb.flush();
+    force_filter(A, T, W, prec, in_prec(phi, 0));
   } else if (T.d.kind == PFMP_KIND_FILTERCORR) {
-    multishift(A, W, T.sig, phi32, PFMP_F32);
-    ForceBatch fb(A, PFMP_F32);
-    for (size_t k = 0; k < T.sig.size(); ++k) {
-      void* chib = fb.ring((int)k);
-      caxpby(c, PFMP_F32, T.r[k], A->xs32[k], 0.0, chib);
-      fb.add_K(W, A->xs32[T.conj_of[k]], chib, -1.0);
-    }
-    fb.flush();
+    multishift(A, W, T.sig, in_prec(phi, 0), prec);
+    std::vector<const void*> x;
+    for (size_t k = 0; k < T.sig.size(); ++k) x.push_back(f32 ? (const void*)A->xs32[k] : (const void*)A->xs[k]);
+    force_filtercorr(A, T, W, prec, x);
   } else if (T.d.kind == PFMP_KIND_RATIO) {
     pfmp_op* Mb = A->ops[T.d.b];
     mhat(W, PFMP_F64, E(A, 0), phi, true, nullptr, nullptr);
-    cg_tol(A, Mb, E(A, 1), E(A, 0), md_tol(A));
-    float4* chi32 = E32(A, 1);
-    blas_copy(c, chi32, PFMP_F32, E(A, 1), PFMP_F64);
-    ForceBatch fb(A, PFMP_F32);
-    fb.add_mhat(W, phi32, chi32, 2.0);
-    fb.add_K(Mb, chi32, chi32, -1.0);
-    fb.flush();
+    cg_tol(A, Mb, E(A, 1), E(A, 0), tol);
+    const void* p = in_prec(phi, 0);
+    force_ratio(A, W, Mb, prec, p, in_prec(E(A, 1), 1));
   } else {  // INV
-    cg_tol(A, W, E(A, 1), phi, md_tol(A));
-    float4* chi32 = E32(A, 1);
-    blas_copy(c, chi32, PFMP_F32, E(A, 1), PFMP_F64);
-    ForceBatch fb(A, PFMP_F32);
-    fb.add_K(W, chi32, chi32, -1.0);
-    fb.flush();
+    cg_tol(A, W, E(A, 1), phi, tol);
+    force_inv(A, W, prec, in_prec(E(A, 1), 1));
   }
 }
 
@@ -637,58 +738,10 @@ void action_force(pfmp_action* A, int i) {
   if (T.d.kind == PFMP_KIND_DET && !clover) return;
   PFMP_CUDA(cudaMemsetAsync(A->Hc, 0, (size_t)g.Vh * 96 * sizeof(double), c->stream));
   void* phi = T.pf >= 0 ? A->phi[T.pf] : nullptr;
-  if (T.d.kind != PFMP_KIND_DET && f32_forces(A)) {
-    force_f32(A, T, W, phi);
-  } else if (T.d.kind == PFMP_KIND_DET) {
+  if (T.d.kind == PFMP_KIND_DET)
     clover_insert_det(W, A->Hc, 2.0 * W->kappa * W->csw);
-  } else if (T.d.kind == PFMP_KIND_FILTER) {
-    const int m = (int)T.q.size();
-    // chi_i, i = m-1 .. 0 (0-based): chi[m-1] = c phi, chi[i] = (J - q_{i+1}) chi[i+1]
-    while ((int)A->xs.size() < m) A->xs.push_back((double2*)dev_alloc(spb(A)));
-    caxpby(c, T.c, phi, 0.0, A->xs[m - 1]);
-    for (int k = m - 2; k >= 0; --k) {
-      kop(W, PFMP_F64, A->xs[k], A->xs[k + 1], nullptr, nullptr);
-      caxpby(c, -T.q[k + 1], A->xs[k + 1], 1.0, A->xs[k]);
-    }
-    // eta_0 = phi, eta_i = (J - q_{i-1}^*) eta_{i-1}, each in its own ring field
-    ForceBatch fb(A, PFMP_F64);
-    const void* eta = phi;
-    for (int k = 0; k < m; ++k) {
-      if (k > 0) {
-        void* next = fb.ring(k);
-        kop(W, PFMP_F64, next, eta, nullptr, nullptr);
-        caxpby(c, -std::conj(T.q[k - 1]), eta, 1.0, next);
-        eta = next;
-      }
-      fb.add_K(W, eta, A->xs[k], 1.0);
-    }
-    fb.flush();
-  } else if (T.d.kind == PFMP_KIND_FILTERCORR) {
-    multishift(A, W, T.sig, phi);
-    ForceBatch fb(A, PFMP_F64);
-    for (size_t k = 0; k < T.sig.size(); ++k) {
-      void* chib = fb.ring((int)k);
-      caxpby(c, T.r[k], A->xs[k], 0.0, chib);
-      fb.add_K(W, A->xs[T.conj_of[k]], chib, -1.0);
-    }
-    fb.flush();
-  } else if (T.d.kind == PFMP_KIND_RATIO) {
-    pfmp_op* Mb = A->ops[T.d.b];
-    mhat(W, PFMP_F64, E(A, 0), phi, true, nullptr, nullptr);
-    void* chi = E(A, 1);
-    cg64(A, Mb, chi, E(A, 0));
-    // 2 Re chi^dag dW^dag phi = 2 Re phi^dag dW chi
-    ForceBatch fb(A, PFMP_F64);
-    fb.add_mhat(W, phi, chi, 2.0);
-    fb.add_K(Mb, chi, chi, -1.0);
-    fb.flush();
-  } else {  // INV
-    void* chi = E(A, 1);
-    cg64(A, W, chi, phi);
-    ForceBatch fb(A, PFMP_F64);
-    fb.add_K(W, chi, chi, -1.0);
-    fb.flush();
-  }
+  else
+    fermion_force(A, T, W, phi);
   if (clover) clover_force(c, fprec, A->F, A->Hc);
 }
 
