@@ -10,7 +10,12 @@
 // Addition is the "sloppy" df add (TwoSum of the high parts, low parts added, one
 // renormalisation): its error is bounded by a few df ulps of |x| + |y|, which is what a
 // stencil sum of many terms needs.  Multiplication is TwoProd of the high parts plus the
-// cross terms, renormalised.
+// cross terms.  Products and the running sums of multiply-adds are not renormalised: the low
+// part of such a sum holds the rounding errors of its few terms, some 2^-24 of the largest
+// partial result, and is itself rounded at 2^-48 of that, as a renormalised one would be.
+// 12 FP32 instructions per multiply-add (18 with two renormalisations).  GB300, r = b - K x with
+// its copies, before / now: 16^3x32 372 / 283 us, 32^3x64 4310 / 3312 us; |r_df - r_f64| / |K x|
+// at 32^3x64 4.8e-15 / 4.3e-15.
 #pragma once
 #include "fields.cuh"
 #include "mad.cuh"
@@ -53,10 +58,13 @@ __device__ __forceinline__ df operator*(df x, df y) {
   float e = __fmaf_rn(x.hi, y.hi, -p);
   e = __fmaf_rn(x.hi, y.lo, e);
   e = __fmaf_rn(x.lo, y.hi, e);
-  return df_fast_two_sum(p, e);
+  return df(p, e);
 }
 
-__device__ __forceinline__ df mad(df x, df y, df z) { return z + x * y; }
+__device__ __forceinline__ df mad(df x, df y, df z) {
+  const df p = x * y, s = df_two_sum(z.hi, p.hi);
+  return df(s.hi, __fadd_rn(z.lo, __fadd_rn(s.lo, p.lo)));
+}
 
 template <>
 struct Prec<2> {  // double-float, used only inside the library (the true residual)
@@ -69,7 +77,10 @@ struct Prec<2> {  // double-float, used only inside the library (the true residu
 constexpr int PREC_DF = 2;
 
 __device__ __forceinline__ cplx<df> c_of(float4 v) { return mk(df(v.x, v.y), df(v.z, v.w)); }
-__device__ __forceinline__ float4 v_of(cplx<df> c) { return make_float4(c.re.hi, c.re.lo, c.im.hi, c.im.lo); }
+__device__ __forceinline__ float4 v_of(cplx<df> c) {
+  const df re = df_fast_two_sum(c.re.hi, c.re.lo), im = df_fast_two_sum(c.im.hi, c.im.lo);
+  return make_float4(re.hi, re.lo, im.hi, im.lo);
+}
 
 template <bool CG = false>
 __device__ __forceinline__ void load_spinor(Spinor<df>& s, const float4* __restrict__ f, int cb, int Vh) {
