@@ -20,14 +20,14 @@ namespace pfmp {
 
 namespace {
 
-// resident 128-thread blocks per SM: 7 as the FP32 stencil; 6 for the two kernels that
-// also carry CG vectors (at 7 they spill 0.1-0.6 KB per thread)
-constexpr int kMinBlocks = 7;
-constexpr int kMinBlocksVec = 6;
+// resident 128-thread blocks per SM (MINB): as the FP32 stencil (resident_blocks), but 6 in
+// place of 7 for the two kernels that also carry CG vectors (at 7 they spill 0.1-0.6 KB per
+// thread)
 
 __device__ __forceinline__ float4 f4(const cplx<float>& a, const cplx<float>& b) { return make_float4(a.re, a.im, b.re, b.im); }
 
-__global__ void __launch_bounds__(128, kMinBlocks) k_cgf_1(HopParams<PFMP_F32> a) {
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_cgf_1(HopParams<PFMP_F32> a) {
   if (a.scal->done) return;
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   if (cb >= a.g.Vh) return;
@@ -36,7 +36,8 @@ __global__ void __launch_bounds__(128, kMinBlocks) k_cgf_1(HopParams<PFMP_F32> a
   store_spinor(a.out, out, cb, a.g.Vh);
 }
 
-__global__ void __launch_bounds__(128, kMinBlocksVec) k_cgf_2(HopParams<PFMP_F32> a, const float4* __restrict__ r,
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_cgf_2(HopParams<PFMP_F32> a, const float4* __restrict__ r,
                                                            float4* __restrict__ p) {
   CGScalars* sc = a.scal;
   if (sc->done) return;
@@ -72,14 +73,16 @@ __global__ void __launch_bounds__(128, kMinBlocksVec) k_cgf_2(HopParams<PFMP_F32
   }
 }
 
-__global__ void __launch_bounds__(128, kMinBlocks) k_cgf_3(HopParams<PFMP_F32> a) {
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_cgf_3(HopParams<PFMP_F32> a) {
   if (a.scal->done) return;
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   if (cb >= a.g.Vh) return;
   store_spinor(a.out, hop_site<PFMP_F32, true, EPI_CLOV>(a, cb), cb, a.g.Vh);
 }
 
-__global__ void __launch_bounds__(128, kMinBlocksVec) k_cgf_4(HopParams<PFMP_F32> a, float4* __restrict__ x,
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_cgf_4(HopParams<PFMP_F32> a, float4* __restrict__ x,
                                                            float4* __restrict__ r, const float4* __restrict__ p) {
   CGScalars* sc = a.scal;
   if (sc->done) return;
@@ -137,9 +140,8 @@ double reals_per_site(int phase) {
 
 }  // namespace
 
-// one fused FP32 CG iteration on the context's stream; x, r, p: FP32 even fields (p holds
-// the previous direction, r the current residual, beta in op->scal the pending step)
-void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
+template <int MINB, int MINB_VEC>
+static void fused_iteration_t(pfmp_op* op, float4* x, float4* r, float4* p) {
   pfmp_ctx* c = op->ctx;
   const Geom& g = c->g;
   const int bs = op->hop_block;
@@ -158,7 +160,7 @@ void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
   a.clov = op->clov32[1];
   a.coef = 1.0;
   prof_start(c, &ev);
-  k_cgf_1<<<grid, bs, 0, c->stream>>>(a);
+  k_cgf_1<MINB><<<grid, bs, 0, c->stream>>>(a);
   PFMP_CHECK_LAUNCH();
   prof_stop(c, PFMP_KERNEL_CG_F32, reals_per_site(1) * 4.0 * g.Vh, ev);
   // phase 2
@@ -169,7 +171,7 @@ void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
   a.clov = op->clov32[0];
   a.coef = -op->kappa * op->kappa;
   prof_start(c, &ev);
-  k_cgf_2<<<grid, bs, 0, c->stream>>>(a, r, p);
+  k_cgf_2<MINB_VEC><<<grid, bs, 0, c->stream>>>(a, r, p);
   PFMP_CHECK_LAUNCH();
   prof_stop(c, PFMP_KERNEL_CG_F32, reals_per_site(2) * 4.0 * g.Vh, ev);
   // phase 3
@@ -179,7 +181,7 @@ void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
   a.clov = op->clov32[1];
   a.coef = 1.0;
   prof_start(c, &ev);
-  k_cgf_3<<<grid, bs, 0, c->stream>>>(a);
+  k_cgf_3<MINB><<<grid, bs, 0, c->stream>>>(a);
   PFMP_CHECK_LAUNCH();
   prof_stop(c, PFMP_KERNEL_CG_F32, reals_per_site(3) * 4.0 * g.Vh, ev);
   // phase 4
@@ -190,10 +192,20 @@ void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
   a.clov = op->clov32[0];
   a.coef = -op->kappa * op->kappa;
   prof_start(c, &ev);
-  k_cgf_4<<<grid, bs, 0, c->stream>>>(a, x, r, p);
+  k_cgf_4<MINB_VEC><<<grid, bs, 0, c->stream>>>(a, x, r, p);
   PFMP_CHECK_LAUNCH();
   prof_stop(c, PFMP_KERNEL_CG_F32, reals_per_site(4) * 4.0 * g.Vh, ev);
   op->kapply += 1;
+}
+
+// one fused FP32 CG iteration on the context's stream; x, r, p: FP32 even fields (p holds
+// the previous direction, r the current residual, beta in op->scal the pending step)
+void cg_fused_iteration(pfmp_op* op, float4* x, float4* r, float4* p) {
+  switch (resident_blocks(op->ctx->g.Vh, 7)) {
+    case 2: fused_iteration_t<2, 2>(op, x, r, p); break;
+    case 4: fused_iteration_t<4, 4>(op, x, r, p); break;
+    default: fused_iteration_t<7, 6>(op, x, r, p);
+  }
 }
 
 }  // namespace pfmp

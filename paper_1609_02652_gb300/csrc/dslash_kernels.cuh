@@ -27,25 +27,28 @@ namespace pfmp {
 // few spilled registers (FP32, 32^3x64: 0.85 -> 0.89 of the copy bandwidth at 7 blocks).
 // The FP16-storage stencil does more arithmetic per byte and runs best with a few more
 // registers (K at 32^3x64: 97.4 us per launch at 7 blocks, 93.1 at 6 or 5, 103 at 8).
-template <int PREC>
+// With a sum the FP32 stencil loops over sites and spills 0.4 KB at 7 blocks: 6.
+template <int PREC, bool REDUCE>
 constexpr int hop_min_blocks() {
   static_assert(PREC == PFMP_F32 || PREC == PFMP_H16, "FP64 and double-float: hop_tile.cuh");
-  return PREC == PFMP_F32 ? 7 : 6;
+  return PREC == PFMP_F32 && !REDUCE ? 7 : 6;
 }
 
-template <int PREC, bool DAG, int EPI, bool REDUCE>
-__global__ void __launch_bounds__(128, hop_min_blocks<PREC>()) k_hop(HopParams<PREC> a) {
+template <int PREC, bool DAG, int EPI, bool REDUCE, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_hop(HopParams<PREC> a) {
   if (a.scal && a.scal->done) return;
-  const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   double nrm[1] = {0.0};
-  if (cb < a.g.Vh) {
+  // with a sum, a block takes sites in turn (see launch_site); without, each thread has one
+  const int step = REDUCE ? gridDim.x * blockDim.x : a.g.Vh;
+  for (int cb = blockIdx.x * blockDim.x + threadIdx.x; cb < a.g.Vh; cb += step) {
     Spinor<typename Prec<PREC>::real> out;
     if constexpr (PREC == PFMP_H16)
       out = hop_site_h16<DAG, EPI>(a, cb);
     else
       out = hop_site<PREC, DAG, EPI>(a, cb);
     store_spinor(a.out, out, cb, a.g.Vh);
-    if (REDUCE) nrm[0] = spinor_norm2(out);
+    if (REDUCE) nrm[0] += spinor_norm2(out);
+    if (!REDUCE) break;
   }
   if (REDUCE) {
     double tot[1];
@@ -101,13 +104,32 @@ int split_of(const pfmp_op* op) {
 }
 
 template <int PREC, bool DAG, int EPI, bool RED>
+void launch_site(const HopParams<PREC>& a, int bs, cudaStream_t st) {
+  constexpr int B = hop_min_blocks<PREC, RED>();
+  const int m = resident_blocks(a.g.Vh, B);
+  int n = nblocks(a.g.Vh, bs);
+  if (RED) {
+    // A block's last act in a sum is a fence and a ticket, about 1.5 us in which its slot does
+    // nothing: the blocks that are resident at once go over the lattice instead (32^3x64, FP16
+    // storage, A_ee x - kappa^2 H t with the norm: 126 -> 99 us; 84 without the norm)
+    const long slots = 152L * m * 128 / bs;
+    n = nblocks(n, (int)((n + slots - 1) / slots));
+  }
+  switch (m) {
+    case 2: k_hop<PREC, DAG, EPI, RED, 2><<<n, bs, 0, st>>>(a); break;
+    case 4: k_hop<PREC, DAG, EPI, RED, 4><<<n, bs, 0, st>>>(a); break;
+    default: k_hop<PREC, DAG, EPI, RED, B><<<n, bs, 0, st>>>(a);
+  }
+}
+
+template <int PREC, bool DAG, int EPI, bool RED>
 void launch(const HopParams<PREC>& a, pfmp_op* op) {
   pfmp_ctx* c = op->ctx;
   cudaEvent_t ev;
   prof_start(c, &ev);
   const int bs = op->hop_block;
   if constexpr (PREC == PFMP_H16) {  // one thread per site only
-    k_hop<PREC, DAG, EPI, RED><<<nblocks(a.g.Vh, bs), bs, 0, c->stream>>>(a);
+    launch_site<PREC, DAG, EPI, RED>(a, bs, c->stream);
   } else {
     const int ns = split_of<PREC>(op);
     const long n = (long)a.g.Vh * ns;
@@ -118,7 +140,7 @@ void launch(const HopParams<PREC>& a, pfmp_op* op) {
       default:
         if constexpr (PREC == PFMP_F32) {
           if (!hop_shared_f32(a.g.Vh)) {
-            k_hop<PREC, DAG, EPI, RED><<<nblocks(a.g.Vh, bs), bs, 0, c->stream>>>(a);
+            launch_site<PREC, DAG, EPI, RED>(a, bs, c->stream);
             break;
           }
         }

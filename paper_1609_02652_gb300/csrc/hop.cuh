@@ -32,6 +32,22 @@ struct HopParams {
   CGScalars* scal;   // optional: alpha = rr / ||out||^2; skip all work once done
 };
 
+// Register bound (resident 128-thread blocks per SM) of the one-thread-per-site FP32 and FP16
+// stencils for Vh sites, `most` where the lattice fills the SMs many times.  A thread has 90
+// 16-byte loads to make; the fewer blocks an SM gets, the more registers it can spare to keep
+// them in flight (255 at 2, 128 at 4, 72 at 7).  4 is taken where its whole waves of blocks
+// cover the lattice with a tenth fewer slots.  GB300, FP32, us per K with a bound of 7 / 4 / 2:
+// 16^4 (1.7 blocks per SM) 37.0 / 32.9 / 29.8, 16^3x24 (2.5) 41.0 / 36.9 / 41.1, 16^3x32 (3.4)
+// 50.6 / 43.9 / 49.2, 18^3x36 (5.4) 80 / 88 / 85, 16^2x24x48 (7.6) 130 / 108 / 118, 24^3x48 (17)
+// 227 / 222 / 241; mixed solve at 4^3x8 2.29 / 2.01 / 1.83 ms, at 16^3x32 5.60 / 5.29 / 5.79.
+inline int resident_blocks(int Vh, int most) {
+  constexpr int kSMs = 152;
+  const int n = nblocks(Vh, 128), per_sm = nblocks(n, kSMs);
+  if (per_sm <= 2) return 2;
+  const int at4 = 4 * nblocks(n, 4 * kSMs), at_most = most * nblocks(n, most * kSMs);
+  return 10 * at4 <= 9 * at_most ? 4 : most;
+}
+
 // the stencil's input at site n: a.in, or with XPY a.in + beta a.in2 (a CG direction
 // p = r + beta p_old formed where the stencil reads it)
 template <int PREC, bool CG, bool XPY>
@@ -571,6 +587,15 @@ __device__ __forceinline__ double spinor_norm2(const Spinor<T>& v) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) t += (double)norm2(v.s[s][c]);
   return t;
+}
+// FP32: the site's twelve terms as a pair sum, as exact as in FP64 without its pipe
+__device__ __forceinline__ double spinor_norm2(const Spinor<float>& v) {
+  PairSum t;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) t.add(norm2(v.s[s][c]));
+  return t.value();
 }
 
 }  // namespace pfmp

@@ -403,15 +403,15 @@ __global__ void __launch_bounds__(8 * kPairSites, 5) k_hop_pair(HopParams<PREC> 
 // ---------------------------------------------------------------- host
 // Several threads per site below, one thread per site from these sizes on (sites per
 // parity; us per K of four launches, GB300):
-//  * FP32: k_hop gives no SM more than one 128-site block until Vh exceeds 128 x 152, and
-//    then waits for one thread's chain of eight neighbours.  k_hop_pair against k_hop:
-//    16.8 / 33.1 at 256, 25.0 / 33.3 at 10368, 33.3 / 37.3 at 20736, 37.3 / 38.7 at 27648,
-//    90 / 50 at 65536.
+//  * FP32: a lattice with few sites leaves k_hop's 128-site blocks on a few SMs, each waiting
+//    for one thread's chain of eight neighbours.  k_hop_pair against k_hop (255 registers):
+//    16.5 / 24.7 at 256 to 2048, 17.2 / 24.7 at 4096, 24.7 / 24.6 at 6144, 32.9 / 24.6 at 20736,
+//    41.0 / 28.8 at 27648.
 //  * FP64 and double-float, always several threads: k_hop_tile (8-site blocks, 16 threads
 //    per site) while the 16-site blocks of k_hop_pair would leave SMs idle, k_hop_pair from
 //    there on.  FP64 tile / pair: 25 / 41 at 128, 33 / 41 at 2048, 58 / 50 at 4096, 545 /
 //    506 at 65536; double-float (true residual) 69 / 77 at 128, 334 / 321 at 65536.
-constexpr int kPairMaxF32 = 160 * 152;
+constexpr int kPairMaxF32 = 32 * 152;
 constexpr int kTileMax = kPairSites * 152;
 inline bool hop_shared_f32(int Vh) { return Vh <= kPairMaxF32; }
 
