@@ -2,13 +2,15 @@
 //
 // Many independent systems K_s x_{s,r} = b_{s,r} (different lattices, gauge fields and
 // kappa; R_s right-hand sides each) are solved by ONE cooperative kernel whose blocks
-// stay resident for the whole solve.  Each phase's work is cut into tiles (system, site
-// block, rhs), the R_s tiles of one site block adjacent so that their link and clover
-// reads share the L2; the blocks take the tiles in turn, and a grid barrier separates
-// the phases.  A CG iteration of the whole batch is six phases: the four stencil phases
-// of K = M-hat^dag M-hat, the x/r update and the p update, each rhs with its own scalars
-// (the per-rhs sums are deterministic: fixed partial slots, summed in a fixed order by
-// the rhs's last tile).  The FP32 iterations are corrected by reliable updates on the
+// stay resident for the whole solve.  Each phase's work is cut into warp tiles (system, 32
+// sites, rhs), the R_s tiles of the same sites adjacent, so that the warps of a block read
+// the same links and clover blocks and L1 serves all but the first: a stencil phase needs
+// 672 bytes of them per site against 192-288 of a rhs's own fields (six systems with
+// 29 rhs: 96 -> 87 ms).  The warps take the tiles in turn, and a grid
+// barrier separates the phases.  A CG iteration of the whole batch is five phases: the four
+// stencil phases of K = M-hat^dag M-hat, the last with the x and r updates in its epilogue,
+// and the p update, each rhs with its own scalars (the per-rhs sums are deterministic: fixed
+// partial slots, summed in a fixed order by the rhs's last tile).  The FP32 iterations are corrected by reliable updates on the
 // device: once a rhs's iterated residual has dropped by delta, x is accumulated in FP64
 // and r = b - K x is recomputed with K in double-float (five more phases, only when some
 // rhs asked for it); a rhs whose double-float residual is below the target stops.  The
@@ -41,7 +43,7 @@ struct PSys {
   double kappa2;
   int R, nsb, rhs0;
   long fw;                          // float4 words of one FP32 half-lattice field (6 Vh)
-  float4 *x, *r, *p, *Ap, *t, *e;   // R FP32 fields each
+  float4 *x, *r, *p, *t, *e;        // R FP32 fields each
   float4 *xdf, *edf, *tdf;          // R double-float fields each (2 fw words)
 };
 
@@ -58,7 +60,7 @@ struct PRhs {
 struct PBatch {
   PSys* sys;
   PRhs* rhs;
-  const int2* tiles;   // (system, site block * R + rhs)
+  const int2* tiles;   // (system, block of 32 sites * R + rhs)
   int ntiles;
   double* partials;    // per rhs: 2 nsb doubles
   unsigned* tickets;   // per rhs
@@ -114,10 +116,40 @@ __device__ bool grid_barrier(const PBatch& B) {
 }
 
 // per-rhs deterministic sum of N values over the rhs's nsb tiles: slot sb of the rhs's
-// partials, the last tile to arrive sums the slots in order (true on its thread 0)
+// partials, the last tile to arrive sums the slots in order (true on its lane 0)
 template <int N>
 __device__ bool rhs_sum(const PBatch& B, const PRhs& R, int idx, int nsb, int sb, double v[N], double out[N]) {
-  return group_sum<N>(v, B.partials + R.part0, B.tickets + idx, (unsigned)nsb, (unsigned)sb, out);
+  const int lane = threadIdx.x & 31;
+  double* part = B.partials + R.part0;
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  bool last = false;
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) part[(size_t)sb * N + k] = v[k];
+    __threadfence();
+    last = atomicAdd(B.tickets + idx, 1u) == (unsigned)nsb - 1;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+  __threadfence();
+  double w[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) w[k] = 0.0;
+#pragma unroll 8
+  for (int b = lane; b < nsb; b += 32)
+#pragma unroll
+    for (int k = 0; k < N; ++k) w[k] += __ldcg(part + (size_t)b * N + k);
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_down_sync(0xffffffffu, w[k], o);
+  if (lane != 0) return false;
+#pragma unroll
+  for (int k = 0; k < N; ++k) out[k] = w[k];
+  B.tickets[idx] = 0u;
+  return true;
 }
 
 __device__ __forceinline__ int ld_state(const PRhs& R) { return *(volatile const int*)&R.state; }
@@ -128,23 +160,54 @@ struct Tile {
   PRhs* R;
   int idx, sb, r, cb;
 };
-__device__ __forceinline__ Tile tile_at(const PBatch& B, int t) {
-  const int2 m = B.tiles[t];
+__device__ __forceinline__ Tile tile_at(const PBatch& B, int2 m) {
   Tile T;
   T.S = B.sys + m.x;
   T.sb = m.y / T.S->R;
   T.r = m.y % T.S->R;
   T.idx = T.S->rhs0 + T.r;
   T.R = B.rhs + T.idx;
-  T.cb = T.sb * blockDim.x + threadIdx.x;
+  T.cb = T.sb * 32 + (threadIdx.x & 31);
   return T;
 }
+// A warp's tiles of one phase, for (Walk w(B); w.more(); w.next()).  The description of a tile and
+// the state of its rhs are two dependent loads from L2 (a rhs's state changes only after its
+// last tile of a phase): they are made two tiles and one tile ahead.
+struct Walk {
+  const PBatch& B;
+  int t;
+  int2 m0, m1, m2;
+  int st0, st1;
+  __device__ __forceinline__ static int step() { return (gridDim.x * blockDim.x) >> 5; }
+  __device__ __forceinline__ int2 get(int i) const { return i < B.ntiles ? __ldg(B.tiles + i) : make_int2(0, 0); }
+  __device__ __forceinline__ int look(int2 m) const {
+    const PSys& S = B.sys[m.x];
+    return ld_state(B.rhs[S.rhs0 + m.y % S.R]);
+  }
+  __device__ __forceinline__ explicit Walk(const PBatch& b) : B(b), t((blockIdx.x * blockDim.x + threadIdx.x) >> 5) {
+    m0 = get(t);
+    m1 = get(t + step());
+    m2 = get(t + 2 * step());
+    st0 = look(m0);
+    st1 = look(m1);
+  }
+  __device__ __forceinline__ bool more() const { return t < B.ntiles; }
+  __device__ __forceinline__ void next() {
+    t += step();
+    m0 = m1;
+    st0 = st1;
+    m1 = m2;
+    st1 = look(m1);
+    m2 = get(t + 2 * step());
+  }
+  __device__ __forceinline__ Tile tile() const { return tile_at(B, m0); }
+};
 
 // ---------------------------------------------------------------- phases
 // b -> r = p (FP32), x = 0 (FP32 and FP64); |b|^2 and |r|^2
 __device__ void phase_init(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
+  for (Walk w(B); w.more(); w.next()) {
+    const Tile T = w.tile();
     const PSys& S = *T.S;
     const int Vh = S.g.Vh;
     const long off = (long)T.r * S.fw;
@@ -168,7 +231,7 @@ __device__ void phase_init(const PBatch& B) {
       v[1] = acc;
     }
     double s[2];
-    if (rhs_sum<2>(B, *T.R, T.idx, S.nsb * 1, T.sb, v, s)) {
+    if (rhs_sum<2>(B, *T.R, T.idx, S.nsb, T.sb, v, s)) {
       PRhs& R = *T.R;
       R.bb = s[0];
       R.rr = s[1];
@@ -190,14 +253,17 @@ __device__ void phase_init(const PBatch& B) {
 }
 
 // the four stencil phases of K (FP32): PHASE 1 t = A_oo^{-1} H_oe v, PHASE 2
-// w = A_ee v - kappa^2 H_eo t with v = p, w = e (DAG false) or v = e, w = Ap (DAG true);
-// the non-adjoint PHASE 2 sums ||e||^2 = <p, K p> and sets alpha
+// A_ee v - kappa^2 H_eo t with v = p (DAG false), stored to e, or v = e (DAG true).  The
+// non-adjoint PHASE 2 sums ||e||^2 = <p, K p> and sets alpha.  The adjoint one has K p of the
+// site in registers: x += alpha p, r -= alpha K p; |r|^2 -> beta, rr; a rhs whose |r|^2 fell
+// below stop_rr (or is not finite) asks for a reliable update
 template <bool DAG, int PHASE>
 __device__ __noinline__ void phase_hop(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
-    if (ld_state(*T.R) != RHS_ITER) continue;
+  for (Walk w(B); w.more(); w.next()) {
+    const Tile T = w.tile();
+    if (w.st0 != RHS_ITER) continue;
     const PSys& S = *T.S;
+    const int Vh = S.g.Vh;
     const long off = (long)T.r * S.fw;
     HopParams<PFMP_F32> a{};
     a.g = S.g;
@@ -213,67 +279,57 @@ __device__ __noinline__ void phase_hop(const PBatch& B) {
       a.p = 0;
       a.in = S.t + off;
       a.x = v;
-      a.out = (DAG ? S.Ap : S.e) + off;
+      a.out = S.e + off;
       a.clov = S.clov32[0];
       a.coef = -S.kappa2;
     }
-    constexpr bool RED = PHASE == 2 && !DAG;
+    constexpr bool LAST = PHASE == 2 && DAG;
     double nrm[1] = {0.0};
-    if (T.cb < S.g.Vh) {
+    if (T.cb < Vh) {
       const auto out = hop_site<PFMP_F32, DAG, PHASE == 1 ? EPI_CLOV : EPI_XPAY, true>(a, T.cb);
-      store_spinor(a.out, out, T.cb, S.g.Vh);
-      if (RED) nrm[0] = spinor_norm2(out);
+      if (!LAST) {
+        store_spinor(a.out, out, T.cb, Vh);
+        if (PHASE == 2) nrm[0] = spinor_norm2(out);
+      } else {
+        const float al = (float)ld_d(T.R->alpha);
+        float acc = 0.f;  // the site's |r|^2 in FP32, across sites in FP64
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const long i = off + (long)k * Vh + T.cb;
+          float4 xx = __ldcg(S.x + i), rr = __ldcg(S.r + i);
+          const float4 pp = __ldcg(S.p + i);
+          const cplx<float> a0 = out.s[(2 * k) / 3][(2 * k) % 3], a1 = out.s[(2 * k + 1) / 3][(2 * k + 1) % 3];
+          xx.x += al * pp.x;
+          xx.y += al * pp.y;
+          xx.z += al * pp.z;
+          xx.w += al * pp.w;
+          rr.x -= al * a0.re;
+          rr.y -= al * a0.im;
+          rr.z -= al * a1.re;
+          rr.w -= al * a1.im;
+          S.x[i] = xx;
+          S.r[i] = rr;
+          acc += rr.x * rr.x + rr.y * rr.y + rr.z * rr.z + rr.w * rr.w;
+        }
+        nrm[0] = acc;
+      }
     }
-    if (RED) {
+    if (PHASE == 2) {
       double s[1];
       if (rhs_sum<1>(B, *T.R, T.idx, S.nsb, T.sb, nrm, s)) {
-        T.R->pAp = s[0];
-        T.R->alpha = ld_d(T.R->rr) / s[0];
-      }
-    }
-  }
-}
-
-// x += alpha p, r -= alpha Ap; |r|^2 -> beta, rr; a rhs whose |r|^2 fell below stop_rr
-// (or is not finite) asks for a reliable update
-__device__ void phase_xr(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
-    if (ld_state(*T.R) != RHS_ITER) continue;
-    const PSys& S = *T.S;
-    const int Vh = S.g.Vh;
-    const long off = (long)T.r * S.fw;
-    const float al = (float)ld_d(T.R->alpha);
-    double v[1] = {0.0};
-    if (T.cb < Vh) {
-      float acc = 0.f;  // the site's |r|^2 in FP32, across sites in FP64
-      for (int k = 0; k < 6; ++k) {
-        const long i = off + (long)k * Vh + T.cb;
-        float4 xx = __ldcg(S.x + i), rr = __ldcg(S.r + i);
-        const float4 pp = __ldcg(S.p + i), aa = __ldcg(S.Ap + i);
-        xx.x += al * pp.x;
-        xx.y += al * pp.y;
-        xx.z += al * pp.z;
-        xx.w += al * pp.w;
-        rr.x -= al * aa.x;
-        rr.y -= al * aa.y;
-        rr.z -= al * aa.z;
-        rr.w -= al * aa.w;
-        S.x[i] = xx;
-        S.r[i] = rr;
-        acc += rr.x * rr.x + rr.y * rr.y + rr.z * rr.z + rr.w * rr.w;
-      }
-      v[0] = acc;
-    }
-    double s[1];
-    if (rhs_sum<1>(B, *T.R, T.idx, S.nsb, T.sb, v, s)) {
-      PRhs& R = *T.R;
-      R.beta = s[0] / ld_d(R.rr);
-      R.rr = s[0];
-      R.iters = *(volatile int*)&R.iters + 1;
-      if (s[0] < ld_d(R.stop_rr) || !(s[0] == s[0]) || !(s[0] < 1e300)) {
-        R.state = RHS_UPDATE;
-        atomicAdd(B.nupd, 1u);
+        PRhs& R = *T.R;
+        if (!DAG) {
+          R.pAp = s[0];
+          R.alpha = ld_d(R.rr) / s[0];
+        } else {
+          R.beta = s[0] / ld_d(R.rr);
+          R.rr = s[0];
+          R.iters = *(volatile int*)&R.iters + 1;
+          if (s[0] < ld_d(R.stop_rr) || !(s[0] == s[0]) || !(s[0] < 1e300)) {
+            R.state = RHS_UPDATE;
+            atomicAdd(B.nupd, 1u);
+          }
+        }
       }
     }
   }
@@ -281,9 +337,9 @@ __device__ void phase_xr(const PBatch& B) {
 
 // p = r + beta p for every rhs that ran this iteration
 __device__ void phase_p(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
-    const int st = ld_state(*T.R);
+  for (Walk w(B); w.more(); w.next()) {
+    const Tile T = w.tile();
+    const int st = w.st0;
     if (st != RHS_ITER && st != RHS_UPDATE) continue;
     const PSys& S = *T.S;
     const int Vh = S.g.Vh;
@@ -300,9 +356,9 @@ __device__ void phase_p(const PBatch& B) {
 
 // reliable update, step 1: x64 += x (FP32), x = 0, xdf = x64 split into FP32 pairs
 __device__ void phase_accumulate(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
-    if (ld_state(*T.R) != RHS_UPDATE) continue;
+  for (Walk w(B); w.more(); w.next()) {
+    const Tile T = w.tile();
+    if (w.st0 != RHS_UPDATE) continue;
     const PSys& S = *T.S;
     const int Vh = S.g.Vh;
     if (T.cb >= Vh) continue;
@@ -331,9 +387,9 @@ __device__ void phase_accumulate(const PBatch& B) {
 // r = b - K x64 in FP64, its FP32 copy, |r|^2 in FP64 and of the FP32 copy
 template <bool DAG, int PHASE>
 __device__ __noinline__ void phase_hop_df(const PBatch& B) {
-  for (int t = blockIdx.x; t < B.ntiles; t += gridDim.x) {
-    const Tile T = tile_at(B, t);
-    if (ld_state(*T.R) != RHS_UPDATE) continue;
+  for (Walk w(B); w.more(); w.next()) {
+    const Tile T = w.tile();
+    if (w.st0 != RHS_UPDATE) continue;
     const PSys& S = *T.S;
     const int Vh = S.g.Vh;
     const long off = 2 * (long)T.r * S.fw;
@@ -446,8 +502,6 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(PBatch B) {
     if (!grid_barrier(B)) return;
     phase_hop<true, 2>(B);
     if (!grid_barrier(B)) return;
-    phase_xr(B);
-    if (!grid_barrier(B)) return;
     phase_p(B);
     if (!grid_barrier(B)) return;
     ++it;
@@ -494,7 +548,7 @@ static void batch_layout(pfmp_batch* B, int block) {
   int idx = 0;
   for (size_t s = 0; s < B->sys.size(); ++s) {
     PSys& S = B->sys[s];
-    S.nsb = (S.g.Vh + block - 1) / block;
+    S.nsb = (S.g.Vh + 31) / 32;
     for (int i = 0; i < S.nsb * S.R; ++i) tiles.push_back(make_int2((int)s, i));
     for (int r = 0; r < S.R; ++r, ++idx) {
       B->h_rhs[idx].part0 = np;
@@ -514,7 +568,7 @@ static void batch_layout(pfmp_batch* B, int block) {
   PFMP_CUDA(cudaGetDevice(&dev));
   PFMP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   PFMP_REQUIRE(per_sm >= 1, PFMP_E_CUDA, "the persistent batch kernel cannot be resident");
-  B->grid = std::min(per_sm * nsm, std::max(B->ntiles, 1));
+  B->grid = std::min(per_sm * nsm, std::max(nblocks(B->ntiles, block / 32), 1));
 }
 
 void batch_destroy(pfmp_batch* B) {
@@ -563,11 +617,11 @@ pfmp_batch* batch_create(int nsys, pfmp_op* const* ops, const int* nrhs) {
       S.R = nrhs[s];
       S.rhs0 = off;
       S.fw = 6L * op->ctx->g.Vh;
-      // 6 FP32 fields and 3 double-float fields (2 words each) per rhs
-      float4* buf = (float4*)dev_alloc((size_t)12 * S.R * S.fw * sizeof(float4));
+      // 5 FP32 fields and 3 double-float fields (2 words each) per rhs
+      float4* buf = (float4*)dev_alloc((size_t)11 * S.R * S.fw * sizeof(float4));
       B->bufs.push_back(buf);
       float4* q = buf;
-      float4** f32[6] = {&S.x, &S.r, &S.p, &S.Ap, &S.t, &S.e};
+      float4** f32[5] = {&S.x, &S.r, &S.p, &S.t, &S.e};
       for (auto f : f32) {
         *f = q;
         q += (size_t)S.R * S.fw;
