@@ -14,6 +14,7 @@
 #include "context.h"
 #include "dfloat.cuh"
 #include "fields.cuh"
+#include "mad.cuh"
 
 namespace pfmp {
 
@@ -24,8 +25,11 @@ __device__ __forceinline__ Mat3<double> mlink(const double2* U, const Geom& g, c
   return M;
 }
 __device__ __forceinline__ void shift(const Geom& g, const int x[4], int mu, int d, int y[4]) {
-  for (int k = 0; k < 4; ++k) y[k] = x[k];
-  y[mu] = (y[mu] + d + g.L[mu]) % g.L[mu];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {  // d = +-1
+    const int v = x[k] + (k == mu ? d : 0);
+    y[k] = v == g.L[k] ? 0 : (v < 0 ? g.L[k] - 1 : v);
+  }
 }
 
 // the link U_mu(x): FP64 from the master field, FP32 from the 12-real compressed copy
@@ -43,7 +47,13 @@ __device__ __forceinline__ Mat3<float> clink<float>(const void* U, const Geom& g
   return M;
 }
 
-// F_{mu nu}(x): traceless part of (Q - Q^dag)/(8i), Q = sum of the four leaves at x
+// F_{mu nu}(x): traceless part of (Q - Q^dag)/(8i), Q = sum of the four leaves at x.  Only Q -
+// Q^dag counts, so a leaf may stand for minus its adjoint, and the leaves pair up on the links
+// U_mu(x) and V = U_mu(x-mu):
+//   Q = U_mu(x) [U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)]
+//     + [U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag - (U_mu(x-mu-nu) U_nu(x-nu))^dag U_nu(x-mu-nu)] V,
+// ten products of fused multiply-adds.  Bound by the FP64 pipe: 24^3x48 12.1 -> 7.0 ms
+// (twelve products, sums of products unfused, before).
 template <typename T>
 __device__ Mat3<T> field_strength(const void* U, const Geom& g, const int x[4], int mu, int nu) {
   int xpm[4], xpn[4], xmm[4], xmn[4], xmmpn[4], xmmmn[4], xpmmn[4];
@@ -54,31 +64,30 @@ __device__ Mat3<T> field_strength(const void* U, const Geom& g, const int x[4], 
   shift(g, xmm, nu, 1, xmmpn);
   shift(g, xmm, nu, -1, xmmmn);
   shift(g, xpm, nu, -1, xpmmn);
-  const Mat3<T> Um = clink<T>(U, g, x, mu), Un = clink<T>(U, g, x, nu);
-  // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-  Mat3<T> Q = matmul_nd(matmul_nd(matmul(Um, clink<T>(U, g, xpm, nu)), clink<T>(U, g, xpn, mu)), Un);
-  // leaf 2: U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag U_mu(x-mu)
-  const Mat3<T> Um_xmm = clink<T>(U, g, xmm, mu);
-  Mat3<T> L = matmul(matmul_nd(matmul_nd(Un, clink<T>(U, g, xmmpn, mu)), clink<T>(U, g, xmm, nu)), Um_xmm);
-  Q = mat_add(Q, L);
-  // leaf 3: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu)
+  auto prod_nd = [](const Mat3<T>& A, const Mat3<T>& B) {  // A B^dag
+    Mat3<T> C = mat_zero<T>();
+    mac_nd(C, A, B);
+    return C;
+  };
+  auto minus = [](Mat3<T> A) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) A.m[i][j] = -A.m[i][j];
+    return A;
+  };
+  const Mat3<T> Un = clink<T>(U, g, x, nu), Un_xmn = clink<T>(U, g, xmn, nu);
+  Mat3<T> Q;
   {
-    Mat3<T> A = dagger(Um_xmm);
-    A = matmul_nd(A, clink<T>(U, g, xmmmn, nu));
-    A = matmul(A, clink<T>(U, g, xmmmn, mu));
-    A = matmul(A, clink<T>(U, g, xmn, nu));
-    L = A;
+    Mat3<T> S = prod_nd(prod_nd(clink<T>(U, g, xpm, nu), clink<T>(U, g, xpn, mu)), Un);
+    mac_dn(S, minus(mm(clink<T>(U, g, xmn, mu), clink<T>(U, g, xpmmn, nu))), Un_xmn);
+    Q = mm(clink<T>(U, g, x, mu), S);
   }
-  Q = mat_add(Q, L);
-  // leaf 4: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x+mu-nu) U_mu(x)^dag
   {
-    Mat3<T> A = dagger(clink<T>(U, g, xmn, nu));
-    A = matmul(A, clink<T>(U, g, xmn, mu));
-    A = matmul(A, clink<T>(U, g, xpmmn, nu));
-    A = matmul_nd(A, Um);
-    L = A;
+    Mat3<T> S = prod_nd(prod_nd(Un, clink<T>(U, g, xmmpn, mu)), clink<T>(U, g, xmm, nu));
+    mac_dn(S, minus(mm(clink<T>(U, g, xmmmn, mu), Un_xmn)), clink<T>(U, g, xmmmn, nu));
+    mac(Q, S, clink<T>(U, g, xmm, mu));
   }
-  Q = mat_add(Q, L);
   Mat3<T> F;
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) {
