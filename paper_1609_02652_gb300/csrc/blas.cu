@@ -24,6 +24,7 @@ __device__ __forceinline__ double dot2(double2 a) { return a.x * a.x + a.y * a.y
 // ---------------------------------------------------------------- elementwise
 // F64 [12][Vh] double2 -> F32 [6][Vh] float4 and back
 __global__ void k_f64_to_f32(const double2* __restrict__ s, float4* __restrict__ d, int Vh) {
+  chain_enter();
   const long n = 6L * Vh;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const long k = i / Vh, cb = i % Vh;
@@ -32,6 +33,7 @@ __global__ void k_f64_to_f32(const double2* __restrict__ s, float4* __restrict__
   }
 }
 __global__ void k_f32_to_f64(const float4* __restrict__ s, double2* __restrict__ d, int Vh, int accumulate) {
+  chain_enter();
   const long n = 6L * Vh;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const long k = i / Vh, cb = i % Vh;
@@ -76,6 +78,7 @@ __device__ __forceinline__ float sq(float4 a) { return a.x * a.x + a.y * a.y + a
 // fraction of the FP32 one), the sums across threads and blocks in FP64
 template <typename V>
 __global__ void k_norm2(const V* __restrict__ x, long n, ReduceBuf rb, double* out) {
+  chain_enter();
   decltype(sq(x[0])) acc = 0;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) acc += sq(x[i]);
   double v[1] = {(double)acc};
@@ -310,16 +313,16 @@ void blas_copy(pfmp_ctx* c, void* dst, int dprec, const void* src, int sprec) {
     PFMP_REQUIRE(dprec == PFMP_F32, PFMP_E_UNSUPPORTED, "FP16 fields are converted to FP32");
     k_h16_to_f32<<<blas_grid(Vh), kBlock, 0, c->stream>>>((const uint4*)src, (float4*)dst, Vh);
   } else if (dprec == PFMP_F32) {
-    k_f64_to_f32<<<blas_grid(6L * Vh), kBlock, 0, c->stream>>>((const double2*)src, (float4*)dst, Vh);
+    launch_chained(k_f64_to_f32, blas_grid(6L * Vh), kBlock, c->stream, (const double2*)src, (float4*)dst, Vh);
   } else {
-    k_f32_to_f64<<<blas_grid(6L * Vh), kBlock, 0, c->stream>>>((const float4*)src, (double2*)dst, Vh, 0);
+    launch_chained(k_f32_to_f64, blas_grid(6L * Vh), kBlock, c->stream, (const float4*)src, (double2*)dst, Vh, 0);
   }
   PFMP_CHECK_LAUNCH();
 }
 
 void blas_add_lo(pfmp_ctx* c, void* x64, const void* x32) {
   const int Vh = c->g.Vh;
-  k_f32_to_f64<<<blas_grid(6L * Vh), kBlock, 0, c->stream>>>((const float4*)x32, (double2*)x64, Vh, 1);
+  launch_chained(k_f32_to_f64, blas_grid(6L * Vh), kBlock, c->stream, (const float4*)x32, (double2*)x64, Vh, 1);
   PFMP_CHECK_LAUNCH();
 }
 
@@ -335,9 +338,9 @@ void blas_axpy(pfmp_ctx* c, int prec, double are, double aim, const void* x, voi
 void blas_norm2(pfmp_ctx* c, int prec, const void* x, double* out_dev) {
   const long n = words(c, prec);
   if (prec == PFMP_F64)
-    k_norm2<double2><<<blas_grid(n), kBlock, 0, c->stream>>>((const double2*)x, n, c->rb, out_dev);
+    launch_chained(k_norm2<double2>, blas_grid(n), kBlock, c->stream, (const double2*)x, n, c->rb, out_dev);
   else
-    k_norm2<float4><<<blas_grid(n), kBlock, 0, c->stream>>>((const float4*)x, n, c->rb, out_dev);
+    launch_chained(k_norm2<float4>, blas_grid(n), kBlock, c->stream, (const float4*)x, n, c->rb, out_dev);
   PFMP_CHECK_LAUNCH();
 }
 

@@ -128,6 +128,7 @@ __device__ __forceinline__ void store_block32(float4* f, const HermBlock<T>& b, 
 // [2 parity][6 plane][9][Vh]
 template <typename T>
 __global__ void k_field_strength(Geom g, const void* __restrict__ U, double* __restrict__ Fout) {
+  chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = blockIdx.y / 6, pl = blockIdx.y % 6;
   if (cb >= g.Vh) return;
@@ -272,6 +273,7 @@ __device__ __forceinline__ bool invert_block(HermBlock<T>& B, double& logdet) {
 template <typename T>
 __global__ void __launch_bounds__(128, 3) k_clover_build(Geom g, const double* __restrict__ Fin, double kc_d,
                                                          CloverOut out, ReduceBuf rb, double* logdet_out) {
+  chain_enter();
   const T kc = (T)kc_d;
   const int p = blockIdx.y;
   double ld[1] = {0.0};
@@ -349,9 +351,9 @@ void field_strength_update(pfmp_ctx* c, int prec) {
   if (!c->fmunu) c->fmunu = (double*)dev_alloc((size_t)c->g.Vh * 2 * 6 * 9 * sizeof(double));
   dim3 grid(nblocks(c->g.Vh, 128), 12);
   if (prec == PFMP_F64)
-    k_field_strength<double><<<grid, 128, 0, c->stream>>>(c->g, c->U64, c->fmunu);
+    launch_chained(k_field_strength<double>, grid, 128, c->stream, c->g, c->U64, c->fmunu);
   else
-    k_field_strength<float><<<grid, 128, 0, c->stream>>>(c->g, c->U32, c->fmunu);
+    launch_chained(k_field_strength<float>, grid, 128, c->stream, c->g, c->U32, c->fmunu);
   PFMP_CHECK_LAUNCH();
   c->fmunu_version = c->gauge_version;
   c->fmunu_prec = prec;
@@ -371,9 +373,9 @@ void clover_build(pfmp_op* op, int fprec) {
   PFMP_CUDA(cudaMemsetAsync(o.bad, 0, sizeof(int), c->stream));
   dim3 grid(std::min(nblocks(2L * c->g.Vh, 128), 152 * 24), 2);
   if (fprec == PFMP_F64)
-    k_clover_build<double><<<grid, 128, 0, c->stream>>>(c->g, c->fmunu, op->kappa * op->csw, o, c->rb, c->d_sums);
+    launch_chained(k_clover_build<double>, grid, 128, c->stream, c->g, c->fmunu, op->kappa * op->csw, o, c->rb, c->d_sums);
   else
-    k_clover_build<float><<<grid, 128, 0, c->stream>>>(c->g, c->fmunu, op->kappa * op->csw, o, c->rb, c->d_sums);
+    launch_chained(k_clover_build<float>, grid, 128, c->stream, c->g, c->fmunu, op->kappa * op->csw, o, c->rb, c->d_sums);
   PFMP_CHECK_LAUNCH();
   PFMP_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, 9 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   PFMP_CUDA(cudaStreamSynchronize(c->stream));

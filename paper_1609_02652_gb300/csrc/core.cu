@@ -79,6 +79,7 @@ __global__ void k_gauge_to_canonical(Geom g, const double2* __restrict__ U, doub
 
 __global__ void k_gauge_compress(Geom g, const double2* __restrict__ U, float4* __restrict__ U32,
                                  float4* __restrict__ Udf, uint4* __restrict__ U16) {
+  chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int pm = blockIdx.y;  // parity*4 + mu
   if (cb >= g.Vh) return;
@@ -175,7 +176,7 @@ static double* canon_scratch(pfmp_ctx* c, size_t doubles) {
 
 void gauge_refresh_compressed(pfmp_ctx* c) {
   dim3 grid(nblocks(c->g.Vh), 8);
-  k_gauge_compress<<<grid, kBlock, 0, c->stream>>>(c->g, c->U64, c->U32, c->Udf, c->U16);
+  launch_chained(k_gauge_compress, grid, kBlock, c->stream, c->g, c->U64, c->U32, c->Udf, c->U16);
   PFMP_CHECK_LAUNCH();
   c->gauge_version++;
 }

@@ -207,6 +207,7 @@ __device__ __forceinline__ void hop_force_dir(double* F, const void* gauge, cons
 #define FHB 2
 #endif
 __global__ void __launch_bounds__(256, FHB) k_force_hop(double* F, const void* gauge, Geom g, DerivBatch B) {
+  chain_enter();
   const int cb = blockIdx.x * 32 + (threadIdx.x & 31);
   const int w = threadIdx.x >> 5, mu = w & 3, pz = w >> 2;
   if (cb >= g.Vh) return;
@@ -246,6 +247,7 @@ __device__ __forceinline__ void load_half_rt(Half<typename Prec<PREC>::real>& h,
 constexpr int kForceSites = 8, kForceGroups = 4;
 template <int PREC>
 __global__ void __launch_bounds__(32 * kForceGroups) k_force_hop_split(double* F, const void* gauge, Geom g, DerivBatch B) {
+  chain_enter();
   using T = typename Prec<PREC>::real;
   using V = typename Prec<PREC>::vec;
   __shared__ T sh[kForceGroups - 1][36][32];
@@ -370,6 +372,7 @@ __device__ __forceinline__ void clover_insert_pair(double* Hc, const Geom& g, in
 // spinors close together and each thread keeps 16 accumulators live instead of 48.
 template <int PREC>
 __global__ void __launch_bounds__(96) k_clover_insert(double* Hc, Geom g, DerivBatch B) {
+  chain_enter();
   const int cb = blockIdx.x * 32 + (threadIdx.x & 31);
   const int K = threadIdx.x >> 5;
   const int p = blockIdx.y;
@@ -454,6 +457,7 @@ __device__ __forceinline__ int d_index(int nu, int mu) { return nu * 3 + mu - (m
 // mu < nu), [2 parity][12][9][Vh] complex
 template <typename T>
 __global__ void k_clover_d(cplx<T>* __restrict__ D, const void* gauge, const T* __restrict__ Hc, Geom g) {
+  chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = blockIdx.y, q = blockIdx.z, nu = q / 3;
   const int mu = q % 3 + (q % 3 >= nu);
@@ -536,6 +540,7 @@ __device__ __forceinline__ cplx<T> tr_lambda_rt(int a, Get Z) {
 // so the four warps share the fields they read through L1.
 template <typename T, int KIND>
 __global__ void __launch_bounds__(128, 4) k_leaf_force(double* F, const void* gauge, const cplx<T>* D, Geom g, double coef) {
+  chain_enter();
   const int cb = blockIdx.x * 32 + (threadIdx.x & 31);
   const int mu = threadIdx.x >> 5;
   const int p = blockIdx.y;
@@ -636,7 +641,7 @@ static void leaf_force(pfmp_ctx* c, double* F, const void* gauge, const cplx<T>*
     if (force_small(c->g))
       k_leaf_force_split<T, KIND><<<split, 24 * kLeafSites, 0, c->stream>>>(F, gauge, D, c->g, coef);
     else
-      k_leaf_force<T, KIND><<<dim3(nblocks(c->g.Vh, 32), 2), 128, 0, c->stream>>>(F, gauge, D, c->g, coef);
+      launch_chained(k_leaf_force<T, KIND>, dim3(nblocks(c->g.Vh, 32), 2), 128, c->stream, F, gauge, D, c->g, coef);
   }
   PFMP_CHECK_LAUNCH();
 }
@@ -654,15 +659,15 @@ void deriv_mhat_batch(pfmp_ctx* c, int prec, double* F, double* Hc, const DerivB
   if (prec == PFMP_F64)
     k_force_hop_split<PFMP_F64><<<split, 32 * kForceGroups, 0, c->stream>>>(F, c->U64, c->g, C);
   else if (force_small(c->g))
-    k_force_hop_split<PFMP_F32><<<split, 32 * kForceGroups, 0, c->stream>>>(F, c->U32, c->g, C);
+    launch_chained(k_force_hop_split<PFMP_F32>, split, 32 * kForceGroups, c->stream, F, c->U32, c->g, C);
   else
-    k_force_hop<<<nblocks(c->g.Vh, 32), 256, 0, c->stream>>>(F, c->U32, c->g, C);
+    launch_chained(k_force_hop, nblocks(c->g.Vh, 32), 256, c->stream, F, c->U32, c->g, C);
   PFMP_CHECK_LAUNCH();
   if (!clover) return;
   if (prec == PFMP_F64)
     k_clover_insert<PFMP_F64><<<grid, 96, 0, c->stream>>>(Hc, c->g, B);
   else
-    k_clover_insert<PFMP_F32><<<grid, 96, 0, c->stream>>>(Hc, c->g, B);
+    launch_chained(k_clover_insert<PFMP_F32>, grid, 96, c->stream, Hc, c->g, B);
   PFMP_CHECK_LAUNCH();
 }
 void clover_insert_det(pfmp_op* op, double* Hc, double coef) {
@@ -689,7 +694,7 @@ void clover_force(pfmp_ctx* c, int prec, double* F, const double* Hc) {
     cplx<float>* D = (cplx<float>*)c->clov_d[1];
     k_to_f32<<<std::min(nblocks(n), 152 * 8), kBlock, 0, c->stream>>>(Hc, c->hc32, n);
     PFMP_CHECK_LAUNCH();
-    k_clover_d<float><<<grid, 64, 0, c->stream>>>(D, c->U32, c->hc32, c->g);
+    launch_chained(k_clover_d<float>, grid, 64, c->stream, D, c->U32, c->hc32, c->g);
     PFMP_CHECK_LAUNCH();
     leaf_force<float, LEAF_CLOVER>(c, F, c->U32, D, 0.0625);
   }

@@ -323,6 +323,7 @@ __device__ __forceinline__ void pair_term(cplx<typename Prec<PREC>::real> sm[3],
 
 template <int PREC, bool DAG, int EPI, bool REDUCE>
 __global__ void __launch_bounds__(8 * kPairSites, 5) k_hop_pair(HopParams<PREC> a) {
+  if constexpr (PREC == PFMP_F32) chain_enter();
   using T = typename Prec<PREC>::real;
   constexpr int NS = kPairSites;
   if (a.scal && a.scal->done) return;
@@ -426,7 +427,11 @@ void launch_shared(const HopParams<PREC>& a, cudaStream_t st) {
   }
   // the kernel loops over its site blocks, so the grid stays within the reduction buffer
   const int n = nblocks(Vh, kPairSites);
-  k_hop_pair<PREC, DAG, EPI, RED><<<n < kMaxReduceBlocks ? n : kMaxReduceBlocks, 8 * kPairSites, 0, st>>>(a);
+  const int blocks = n < kMaxReduceBlocks ? n : kMaxReduceBlocks;
+  if constexpr (PREC == PFMP_F32)
+    launch_chained(k_hop_pair<PREC, DAG, EPI, RED>, blocks, 8 * kPairSites, st, a);
+  else
+    k_hop_pair<PREC, DAG, EPI, RED><<<blocks, 8 * kPairSites, 0, st>>>(a);
 }
 
 }  // namespace pfmp

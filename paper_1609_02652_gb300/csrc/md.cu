@@ -46,6 +46,7 @@ void spinor_pack_any(pfmp_ctx* c, void* dst, int prec, const double* src, int wh
 
 // ------------------------------------------------------------------ kernels
 __global__ void k_mom_update(double* __restrict__ p, const double* __restrict__ F, double eps, long n) {
+  chain_enter();
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) p[i] -= eps * F[i];
 }
 
@@ -58,6 +59,7 @@ __global__ void k_sumsq(const double* __restrict__ p, long n, ReduceBuf rb, doub
 
 // U <- exp(i eps P) U, P = sum_a p_a T_a, then reunitarise (FP64 master field)
 __global__ void k_link_update(double2* U, const double* __restrict__ mom, Geom g, double eps) {
+  chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int pm = blockIdx.y;  // parity * 4 + mu
   if (cb >= g.Vh) return;
@@ -105,6 +107,7 @@ static int grid_for(long n) {
 // independent of scheduling); *maxbits must be zero on entry
 __global__ void k_force_norm(const double* __restrict__ F, int Vh, ReduceBuf rb, double* out,
                              unsigned long long* maxbits) {
+  chain_enter();
   double v[1] = {0.0};
   double mx = 0.0;
   const long nl = 8L * Vh;
@@ -803,7 +806,7 @@ double kinetic(pfmp_action* A) {
 void link_update(pfmp_action* A, double eps) {
   pfmp_ctx* c = A->ctx;
   dim3 grid(nblocks(c->g.Vh, 128), 8);
-  k_link_update<<<grid, 128, 0, c->stream>>>(c->U64, A->mom, c->g, eps);
+  launch_chained(k_link_update, grid, 128, c->stream, c->U64, A->mom, c->g, eps);
   PFMP_CHECK_LAUNCH();
   gauge_refresh_compressed(c);
   refresh_ops(A, f32_forces(A) ? PFMP_F32 : PFMP_F64);
@@ -812,7 +815,7 @@ void link_update(pfmp_action* A, double eps) {
 void mom_update(pfmp_action* A, double eps) {
   pfmp_ctx* c = A->ctx;
   const long n = 64L * c->g.Vh;
-  k_mom_update<<<grid_for(n), kBlock, 0, c->stream>>>(A->mom, A->F, eps, n);
+  launch_chained(k_mom_update, grid_for(n), kBlock, c->stream, A->mom, A->F, eps, n);
   PFMP_CHECK_LAUNCH();
 }
 
@@ -821,7 +824,7 @@ void force_norms(pfmp_action* A, double* sum, double* mx) {
   pfmp_ctx* c = A->ctx;
   PFMP_CUDA(cudaMemsetAsync(c->d_sums, 0, 2 * sizeof(double), c->stream));
   const long nl = 8L * c->g.Vh;
-  k_force_norm<<<grid_for(nl), kBlock, 0, c->stream>>>(A->F, c->g.Vh, c->rb, c->d_sums,
+  launch_chained(k_force_norm, grid_for(nl), kBlock, c->stream, A->F, c->g.Vh, c->rb, c->d_sums,
                                                        (unsigned long long*)(c->d_sums + 1));
   PFMP_CHECK_LAUNCH();
   double v[2];

@@ -125,7 +125,8 @@ __device__ __forceinline__ float4 xpby_real(float4 r, double bd, float4 p) {
 // kernel at 24^3x48 with 13 shifts 41 -> 27 us.)
 template <typename V>
 __global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V* __restrict__ Ap, long n, ReduceBuf rb,
-                       CGScalars* s, MSSeed* sd, MSShift* sh, int ns, int* act, int slot) {
+                       CGScalars* s, MSSeed* sd, MSShift* sh, int ns, int* act, int slot, bool chained) {
+  chain_enter(chained);
   if (s->done) {  // a block that starts after the end has no iterations
     if (slot == 0 && blockIdx.x == 0 && threadIdx.x == 0) sd->count = 0;
     return;
@@ -194,7 +195,8 @@ __global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V*
 
 // seed direction p = r + beta p
 template <typename V>
-__global__ void k_ms_p(V* __restrict__ p, const V* __restrict__ r, long n, const CGScalars* s) {
+__global__ void k_ms_p(V* __restrict__ p, const V* __restrict__ r, long n, const CGScalars* s, bool chained) {
+  chain_enter(chained);
   if (s->done) return;
   const double be = s->beta;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
@@ -238,7 +240,8 @@ struct MSRing {
 };
 template <typename V>
 __global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRing<V> ring, const MSShift* __restrict__ sh,
-                                                  const int* __restrict__ act, const MSSeed* sd, long n) {
+                                                  const int* __restrict__ act, const MSSeed* sd, long n, bool chained) {
+  chain_enter(chained);
   using C = typename MSCoef<V>::C;
   const int cnt = sd->count;
   if (cnt == 0) return;
@@ -293,6 +296,7 @@ __global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRi
 // reading y (its previous contents may be anything, NaN included)
 template <typename V>
 __global__ void k_caxpby(double2 a, const V* __restrict__ x, double2 b, V* __restrict__ y, long n) {
+  chain_enter();
   const bool read_y = b.x != 0.0 || b.y != 0.0;
   const double2 zero = make_double2(0.0, 0.0);
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
@@ -311,7 +315,7 @@ void caxpby(pfmp_ctx* c, int prec, std::complex<double> a, const void* x, std::c
   if (prec == PFMP_F64)
     k_caxpby<double2><<<ms_grid(n), kBlock, 0, c->stream>>>(da, (const double2*)x, db, (double2*)y, n);
   else
-    k_caxpby<float4><<<ms_grid(n), kBlock, 0, c->stream>>>(da, (const float4*)x, db, (float4*)y, n);
+    launch_chained(k_caxpby<float4>, ms_grid(n), kBlock, c->stream, da, (const float4*)x, db, (float4*)y, n);
   PFMP_CHECK_LAUNCH();
 }
 void caxpby(pfmp_ctx* c, std::complex<double> a, const void* x, std::complex<double> b, void* y) {
@@ -375,6 +379,7 @@ void ms_work_free(pfmp_op* op) {
 template <typename V>
 static void ms_chunk(pfmp_op* op, int prec, MSWork& w, int ns, void* pseed, void* Ap, long n, int chunk) {
   pfmp_ctx* c = op->ctx;
+  const bool chained = chain_launches(c->stream);
   MSRing<V> ring;
   for (int b = 0; b < kMsBlock; ++b) ring.r[b] = (V*)w.ring[prec == PFMP_F64 ? 0 : 1][b];
   // rows of shifts until the pass has about four blocks per SM
@@ -384,14 +389,14 @@ static void ms_chunk(pfmp_op* op, int prec, MSWork& w, int ns, void* pseed, void
     kop(op, prec, Ap, pseed, &op->scal->pAp, op->scal);
     // the residual before a chunk is in the last slot (every chunk but the last is whole blocks)
     const V* prev = ring.r[slot == 0 ? kMsBlock - 1 : slot - 1];
-    k_ms_r<V><<<nb, kBlock, 0, c->stream>>>(ring.r[slot], prev, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh, ns,
-                                            w.d_act, slot);
+    launch_chained(k_ms_r<V>, nb, kBlock, c->stream, ring.r[slot], prev, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh, ns,
+                                            w.d_act, slot, chained);
     PFMP_CHECK_LAUNCH();
-    k_ms_p<V><<<nb, kBlock, 0, c->stream>>>((V*)pseed, ring.r[slot], n, op->scal);
+    launch_chained(k_ms_p<V>, nb, kBlock, c->stream, (V*)pseed, ring.r[slot], n, op->scal, chained);
     PFMP_CHECK_LAUNCH();
     if (slot == kMsBlock - 1 || k == chunk - 1) {
-      k_ms_xp<V><<<dim3(nb, rows), kBlock, 0, c->stream>>>((V* const*)w.d_x, (V* const*)w.d_p, ring, w.d_sh, w.d_act,
-                                                           w.d_seed, n);
+      launch_chained(k_ms_xp<V>, dim3(nb, rows), kBlock, c->stream, (V* const*)w.d_x, (V* const*)w.d_p, ring, w.d_sh, w.d_act,
+                                                           w.d_seed, n, chained);
       PFMP_CHECK_LAUNCH();
     }
   }

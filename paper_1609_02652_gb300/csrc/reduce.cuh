@@ -6,6 +6,46 @@
 
 namespace pfmp {
 
+// Kernels that follow each other on a stream without the launch gap between them: a kernel
+// launched with launch_chained may become resident while its predecessor drains, and
+// chain_enter, its first statement, waits until the predecessor has completed (its writes
+// are then visible) after letting its own successor come up in the same way.  A successor
+// launched in the ordinary way waits for completion as always.  In a kernel that takes
+// chain_enter, loads through the read-only path come after a branch or inside a loop: in the
+// entry block the compiler could move them above the wait.
+// K at 4^3x8 (four launches of k_hop_pair) 16.4 -> 10.7 us.  The FP64 stencils and force
+// contractions gain nothing (the FP64 force at 6x10x14x18 +2%), nor do the one-thread-per-site
+// stencils (K at 32^3x64 +2%): those are launched in the ordinary way.  Inside a CUDA graph
+// these edges cost more than they hide (mixed solve at 16^3x32 6.1 -> 6.9 ms), so a captured
+// launch is an ordinary one; kernels that run on both sides are told (chained) where they can
+// be without a cost.
+__device__ __forceinline__ void chain_enter() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_enter(bool chained) {
+  if (chained) chain_enter();
+}
+// whether launches on st are chained
+inline bool chain_launches(cudaStream_t st) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  PFMP_CUDA(cudaStreamIsCapturing(st, &capture));
+  return capture == cudaStreamCaptureStatusNone;
+}
+template <typename... P, typename... A>
+void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = chain_launches(st) ? 1 : 0;
+  PFMP_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+}
+
 struct ReduceBuf {
   double* partials;   // [max_blocks * kMaxSums]
   unsigned* counter;  // one ticket counter, left at 0 after each use

@@ -12,11 +12,13 @@
 namespace pfmp {
 
 __global__ void k_split_df(const double2* __restrict__ x, float4* __restrict__ y, long n) {
+  chain_enter();
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) y[i] = split2(x[i]);
 }
 
 __global__ void k_residual_df(const double2* __restrict__ b, const float4* __restrict__ kx, double2* __restrict__ r,
                               long n, ReduceBuf rb, double* out) {
+  chain_enter();
   double v[1] = {0.0};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const double2 bb = b[i];
@@ -36,6 +38,7 @@ static int rgrid(long n) {
 
 // r = b - r, |r|^2 -> *out
 __global__ void k_b_minus_r(const double2* __restrict__ b, double2* __restrict__ r, long n, ReduceBuf rb, double* out) {
+  chain_enter();
   double v[1] = {0.0};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const double2 bb = b[i], kx = r[i];
@@ -50,10 +53,10 @@ __global__ void k_b_minus_r(const double2* __restrict__ b, double2* __restrict__
 double true_residual_df(pfmp_op* op, const void* x64, const void* b64, void* r64) {
   pfmp_ctx* c = op->ctx;
   const long n = 12L * c->g.Vh;
-  k_split_df<<<rgrid(n), kBlock, 0, c->stream>>>((const double2*)x64, op->xdf, n);
+  launch_chained(k_split_df, rgrid(n), kBlock, c->stream, (const double2*)x64, op->xdf, n);
   PFMP_CHECK_LAUNCH();
   kop_df(op, op->kdf, op->xdf);
-  k_residual_df<<<rgrid(n), kBlock, 0, c->stream>>>((const double2*)b64, op->kdf, (double2*)r64, n, c->rb, c->d_sums);
+  launch_chained(k_residual_df, rgrid(n), kBlock, c->stream, (const double2*)b64, op->kdf, (double2*)r64, n, c->rb, c->d_sums);
   PFMP_CHECK_LAUNCH();
   PFMP_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   PFMP_CUDA(cudaStreamSynchronize(c->stream));
@@ -65,7 +68,7 @@ double true_residual_f64(pfmp_op* op, const void* x64, const void* b64, void* r6
   pfmp_ctx* c = op->ctx;
   const long n = 12L * c->g.Vh;
   kop(op, PFMP_F64, r64, x64, nullptr, nullptr);
-  k_b_minus_r<<<rgrid(n), kBlock, 0, c->stream>>>((const double2*)b64, (double2*)r64, n, c->rb, c->d_sums);
+  launch_chained(k_b_minus_r, rgrid(n), kBlock, c->stream, (const double2*)b64, (double2*)r64, n, c->rb, c->d_sums);
   PFMP_CHECK_LAUNCH();
   PFMP_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   PFMP_CUDA(cudaStreamSynchronize(c->stream));
