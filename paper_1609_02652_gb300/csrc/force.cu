@@ -203,10 +203,7 @@ __device__ __forceinline__ void hop_force_dir(double* F, const void* gauge, cons
 // FP32: a block takes 32 sites of both parities; warp (parity, mu) the links of direction mu.
 // The warps of one parity read the same local spinors close together, and one parity's local
 // fields are the other's neighbours, so L1 serves them after the first.
-#ifndef FHB
-#define FHB 2
-#endif
-__global__ void __launch_bounds__(256, FHB) k_force_hop(double* F, const void* gauge, Geom g, DerivBatch B) {
+__global__ void __launch_bounds__(256, 2) k_force_hop(double* F, const void* gauge, Geom g, DerivBatch B) {
   chain_enter();
   const int cb = blockIdx.x * 32 + (threadIdx.x & 31);
   const int w = threadIdx.x >> 5, mu = w & 3, pz = w >> 2;
