@@ -697,8 +697,12 @@ static bool layer_site(pfmp_ctx* c, const void* W, int cin, const void* in, void
   return true;
 }
 
-// packed FP16 weights up to date and kernel attributes set (outside any stream capture)
+// packed FP16 weights up to date and kernel attributes set (outside any stream capture).  The
+// kernels form one sequence, first - hidden ... - last, so a network whose channels return to
+// 1 in between (8 -> 1 -> 8) is refused although each of its layers could be packed.
 static void tc_prepare(pfmp_nn* N) {
+  for (size_t l = 1; l + 1 < N->ch.size(); ++l)
+    PFMP_REQUIRE(N->ch[l] == 8, PFMP_E_INVALID, "tensor-core layer sequence: 1 -> 8 -> ... -> 8 -> 1");
   if (!N->packed) {
     for (size_t l = 0; l < N->W.size(); ++l) nn_tc_pack(N->ctx, N->ch[l], N->ch[l + 1], N->W[l], N->Bp[l]);
     N->packed = true;
