@@ -23,21 +23,21 @@ __device__ __forceinline__ double dot2(double2 a) { return a.x * a.x + a.y * a.y
 
 // ---------------------------------------------------------------- elementwise
 // F64 [12][Vh] double2 -> F32 [6][Vh] float4 and back
-__global__ void k_f64_to_f32(const double2* __restrict__ s, float4* __restrict__ d, int Vh) {
+__global__ void k_f64_to_f32(const double2* s, float4* __restrict__ d, int Vh) {
   chain_enter();
   const long n = 6L * Vh;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const long k = i / Vh, cb = i % Vh;
-    double2 a = s[(2 * k) * Vh + cb], b = s[(2 * k + 1) * Vh + cb];
+    double2 a = ld_live(s + (2 * k) * Vh + cb), b = ld_live(s + (2 * k + 1) * Vh + cb);
     d[i] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
   }
 }
-__global__ void k_f32_to_f64(const float4* __restrict__ s, double2* __restrict__ d, int Vh, int accumulate) {
+__global__ void k_f32_to_f64(const float4* s, double2* __restrict__ d, int Vh, int accumulate) {
   chain_enter();
   const long n = 6L * Vh;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const long k = i / Vh, cb = i % Vh;
-    float4 v = s[i];
+    float4 v = ld_live(s + i);
     double2 a = make_double2(v.x, v.y), b = make_double2(v.z, v.w);
     if (accumulate) {
       double2 a0 = d[(2 * k) * Vh + cb], b0 = d[(2 * k + 1) * Vh + cb];
@@ -77,10 +77,10 @@ __device__ __forceinline__ float sq(float4 a) { return a.x * a.x + a.y * a.y + a
 // FP32 fields: each thread's few terms summed in FP32 (GB300's FP64 pipe is a small
 // fraction of the FP32 one), the sums across threads and blocks in FP64
 template <typename V>
-__global__ void k_norm2(const V* __restrict__ x, long n, ReduceBuf rb, double* out) {
+__global__ void k_norm2(const V* x, long n, ReduceBuf rb, double* out) {
   chain_enter();
   decltype(sq(x[0])) acc = 0;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) acc += sq(x[i]);
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) acc += sq(ld_live(x + i));
   double v[1] = {(double)acc};
   double t[1];
   if (grid_sum<1>(v, rb, t)) *out = t[0];

@@ -20,8 +20,13 @@ namespace pfmp {
 
 __device__ __forceinline__ Mat3<double> mlink(const double2* U, const Geom& g, const int x[4], int mu) {
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+  const double2* f = U + (size_t)((p * 4 + mu) * 9) * g.Vh + cb_index(g, x);
   Mat3<double> M;
-  load_link18(M, U + (size_t)((p * 4 + mu) * 9) * g.Vh, cb_index(g, x), g.Vh);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double2 v = ld_live(f + (size_t)k * g.Vh);
+    M.m[k / 3][k % 3] = mk(v.x, v.y);
+  }
   return M;
 }
 __device__ __forceinline__ void shift(const Geom& g, const int x[4], int mu, int d, int y[4]) {
@@ -32,7 +37,8 @@ __device__ __forceinline__ void shift(const Geom& g, const int x[4], int mu, int
   }
 }
 
-// the link U_mu(x): FP64 from the master field, FP32 from the 12-real compressed copy
+// the link U_mu(x): FP64 from the master field, FP32 from the 12-real compressed copy (both just
+// written by the kernels before this one)
 template <typename T>
 __device__ __forceinline__ Mat3<T> clink(const void* U, const Geom& g, const int x[4], int mu);
 template <>
@@ -43,7 +49,14 @@ template <>
 __device__ __forceinline__ Mat3<float> clink<float>(const void* U, const Geom& g, const int x[4], int mu) {
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
   Mat3<float> M;
-  load_link(M, link_plane<PFMP_F32>((const float4*)U, p * 4 + mu, g.Vh), cb_index(g, x), g.Vh);
+  const float4* f = link_plane<PFMP_F32>((const float4*)U, p * 4 + mu, g.Vh) + cb_index(g, x);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 v = ld_live(f + (size_t)k * g.Vh);
+    M.m[(2 * k) / 3][(2 * k) % 3] = mk(v.x, v.y);
+    M.m[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(v.z, v.w);
+  }
+  reconstruct_row2(M);
   return M;
 }
 
@@ -127,7 +140,7 @@ __device__ __forceinline__ void store_block32(float4* f, const HermBlock<T>& b, 
 // its three diagonal reals and the upper triangle (0,1), (0,2), (1,2), 9 reals per plane,
 // [2 parity][6 plane][9][Vh]
 template <typename T>
-__global__ void k_field_strength(Geom g, const void* __restrict__ U, double* __restrict__ Fout) {
+__global__ void k_field_strength(Geom g, const void* U, double* __restrict__ Fout) {
   chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = blockIdx.y / 6, pl = blockIdx.y % 6;
@@ -150,11 +163,11 @@ __global__ void k_field_strength(Geom g, const void* __restrict__ U, double* __r
 }
 
 template <typename T>
-__device__ __forceinline__ Mat3<T> load_fmunu(const double* __restrict__ Fin, const Geom& g, int p, int pl, int cb) {
+__device__ __forceinline__ Mat3<T> load_fmunu(const double* Fin, const Geom& g, int p, int pl, int cb) {
   const double* f = Fin + (size_t)((p * 6 + pl) * 9) * g.Vh + cb;
   T v[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) v[k] = (T)__ldg(f + (size_t)k * g.Vh);
+  for (int k = 0; k < 9; ++k) v[k] = (T)ld_live(f + (size_t)k * g.Vh);
   Mat3<T> F;
   F.m[0][0] = mk(v[0], T(0));
   F.m[1][1] = mk(v[1], T(0));
@@ -271,7 +284,7 @@ __device__ __forceinline__ bool invert_block(HermBlock<T>& B, double& logdet) {
 // double, or float for the clover terms built from an FP32 field strength inside an MD
 // with FP32 forces (FP32 is all the accuracy such a field strength carries).
 template <typename T>
-__global__ void __launch_bounds__(128, 3) k_clover_build(Geom g, const double* __restrict__ Fin, double kc_d,
+__global__ void __launch_bounds__(128, 3) k_clover_build(Geom g, const double* Fin, double kc_d,
                                                          CloverOut out, ReduceBuf rb, double* logdet_out) {
   chain_enter();
   const T kc = (T)kc_d;

@@ -77,17 +77,17 @@ __global__ void k_gauge_to_canonical(Geom g, const double2* __restrict__ U, doub
   }
 }
 
-__global__ void k_gauge_compress(Geom g, const double2* __restrict__ U, float4* __restrict__ U32,
+__global__ void k_gauge_compress(Geom g, const double2* U, float4* __restrict__ U32,
                                  float4* __restrict__ Udf, uint4* __restrict__ U16) {
   chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int pm = blockIdx.y;  // parity*4 + mu
   if (cb >= g.Vh) return;
   const double2* src = U + (size_t)(pm * 9) * g.Vh;
-  double2 v[6];
-  for (int k = 0; k < 6; ++k) v[k] = src[(size_t)k * g.Vh + cb];
+  double2 v[9];
+  for (int k = 0; k < 9; ++k) v[k] = ld_live(src + (size_t)k * g.Vh + cb);
   float4* ddf = Udf + (size_t)(pm * 9) * g.Vh;
-  for (int k = 0; k < 9; ++k) ddf[(size_t)k * g.Vh + cb] = split2(src[(size_t)k * g.Vh + cb]);
+  for (int k = 0; k < 9; ++k) ddf[(size_t)k * g.Vh + cb] = split2(v[k]);
   float4* d32 = U32 + (size_t)(pm * 3) * g.Vh;
   for (int k = 0; k < 3; ++k)
     d32[(size_t)k * g.Vh + cb] =

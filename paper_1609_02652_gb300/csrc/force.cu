@@ -124,6 +124,23 @@ __device__ __forceinline__ Mat3<typename Prec<PREC>::real> force_link(const void
   }
 }
 
+// the spinor at site cb of a field that the kernels before this one wrote
+__device__ __forceinline__ void load_spinor_live(Spinor<float>& s, const float4* f, int cb, int Vh) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const float4 v = ld_live(f + (size_t)k * Vh + cb);
+    s.s[(2 * k) / 3][(2 * k) % 3] = mk(v.x, v.y);
+    s.s[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(v.z, v.w);
+  }
+}
+__device__ __forceinline__ void load_spinor_live(Spinor<double>& s, const double2* f, int cb, int Vh) {
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const double2 v = ld_live(f + (size_t)k * Vh + cb);
+    s.s[k / 3][k % 3] = mk(v.x, v.y);
+  }
+}
+
 // Spinor products in the arithmetic of PREC (FP64, or FP32 for the MD forces, whose
 // value only has to be a deterministic function of the gauge field).  On the sites of
 // parity pz the forward and backward fields of a contraction (a, b, y, w) are
@@ -182,16 +199,16 @@ __device__ __forceinline__ void hop_force_dir(double* F, const void* gauge, cons
     const T c = (T)(B.c_common == 1.0 ? d.c_hop : 1.0);
     {
       Spinor<T> lf, rf;
-      load_spinor(lf, (const V*)(pz == 0 ? d.a : d.w), cb, g.Vh);
-      load_spinor(rf, (const V*)(pz == 0 ? d.y : d.b), n, g.Vh);
+      load_spinor_live(lf, (const V*)(pz == 0 ? d.a : d.w), cb, g.Vh);
+      load_spinor_live(rf, (const V*)(pz == 0 ? d.y : d.b), n, g.Vh);
       Half<T> l = project<MU, -1>(lf);
       scale_half(l, c);
       outer_half(Xf, project<MU, -1>(rf), l);
     }
     {
       Spinor<T> lb, rb;
-      load_spinor(lb, (const V*)(pz == 0 ? d.w : d.a), n, g.Vh);
-      load_spinor(rb, (const V*)(pz == 0 ? d.b : d.y), cb, g.Vh);
+      load_spinor_live(lb, (const V*)(pz == 0 ? d.w : d.a), n, g.Vh);
+      load_spinor_live(rb, (const V*)(pz == 0 ? d.b : d.y), cb, g.Vh);
       Half<T> r = project<MU, +1>(rb);
       scale_half(r, c);
       outer_half(Xb, r, project<MU, +1>(lb));
@@ -328,8 +345,8 @@ __device__ __forceinline__ void clover_insert_pair(double* Hc, const Geom& g, in
     const DerivSet& d = B.s[s];
     const T coef = (T)(2.0 * (p == 0 ? d.c_even : d.c_odd));
     Spinor<T> a, b;
-    load_spinor(a, (const V*)(p == 0 ? d.a : d.w), cb, g.Vh);
-    load_spinor(b, (const V*)(p == 0 ? d.b : d.y), cb, g.Vh);
+    load_spinor_live(a, (const V*)(p == 0 ? d.a : d.w), cb, g.Vh);
+    load_spinor_live(b, (const V*)(p == 0 ? d.b : d.y), cb, g.Vh);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -432,7 +449,7 @@ __device__ __forceinline__ Mat3<T> load_H(const T* Hc, const Geom& g, const int 
   const int cb = cb_index(g, x);
   T h[8];
 #pragma unroll
-  for (int a = 0; a < 8; ++a) h[a] = sgn * __ldg(Hc + (size_t)((p * 6 + plane) * 8 + a) * g.Vh + cb);
+  for (int a = 0; a < 8; ++a) h[a] = sgn * ld_live(Hc + (size_t)((p * 6 + plane) * 8 + a) * g.Vh + cb);
   return from_algebra<T>(h);
 }
 
@@ -453,7 +470,7 @@ __device__ __forceinline__ int d_index(int nu, int mu) { return nu * 3 + mu - (m
 // D_nu(x) = H(x) U_nu(x) + U_nu(x) H(x+nu) of the 12 ordered planes (sign of H: + for
 // mu < nu), [2 parity][12][9][Vh] complex
 template <typename T>
-__global__ void k_clover_d(cplx<T>* __restrict__ D, const void* gauge, const T* __restrict__ Hc, Geom g) {
+__global__ void k_clover_d(cplx<T>* __restrict__ D, const void* gauge, const T* Hc, Geom g) {
   chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = blockIdx.y, q = blockIdx.z, nu = q / 3;
@@ -473,17 +490,17 @@ __global__ void k_clover_d(cplx<T>* __restrict__ D, const void* gauge, const T* 
 }
 
 template <typename T>
-__device__ __forceinline__ Mat3<T> load_d(const cplx<T>* __restrict__ D, const Geom& g, const int x[4], int nu, int mu) {
+__device__ __forceinline__ Mat3<T> load_d(const cplx<T>* D, const Geom& g, const int x[4], int nu, int mu) {
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
   const cplx<T>* o = D + (size_t)((p * 12 + d_index(nu, mu)) * 9) * g.Vh + cb_index(g, x);
   Mat3<T> M;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     if constexpr (sizeof(T) == 8) {
-      const double2 v = __ldg(reinterpret_cast<const double2*>(o + (size_t)e * g.Vh));
+      const double2 v = ld_live(reinterpret_cast<const double2*>(o + (size_t)e * g.Vh));
       M.m[e / 3][e % 3] = mk(v.x, v.y);
     } else {
-      const float2 v = __ldg(reinterpret_cast<const float2*>(o + (size_t)e * g.Vh));
+      const float2 v = ld_live(reinterpret_cast<const float2*>(o + (size_t)e * g.Vh));
       M.m[e / 3][e % 3] = mk(v.x, v.y);
     }
   }

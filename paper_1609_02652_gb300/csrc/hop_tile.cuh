@@ -45,13 +45,14 @@ __device__ __forceinline__ cplx<T> tile_unit(const cplx<T>& v, bool isI, bool ne
   return isI ? mk(sign_if(v.im, !neg), sign_if(v.re, neg)) : mk(sign_if(v.re, neg), sign_if(v.im, neg));
 }
 
-// complex components 3 s .. 3 s + 2 (spin s) of the spinor at site cb
+// complex components 3 s .. 3 s + 2 (spin s) of the spinor at site cb.  FP32: the kernels that
+// take it are chained (reduce.cuh), so no load of a spinor goes through the read-only path.
 template <int PREC>
 __device__ __forceinline__ void load_spin(cplx<typename Prec<PREC>::real> v[3], const typename Prec<PREC>::vec* f, int s,
                                           int cb, int Vh) {
   if constexpr (PREC == PFMP_F32) {  // two components per word: spin s starts at word 3 s / 2
     const float4* q = f + (size_t)((3 * s) >> 1) * Vh + cb;
-    const float4 a = __ldg(q), b = __ldg(q + Vh);
+    const float4 a = ld_live(q), b = ld_live(q + Vh);
     const bool odd = s & 1;
     v[0] = odd ? mk(a.z, a.w) : mk(a.x, a.y);
     v[1] = odd ? mk(b.x, b.y) : mk(a.z, a.w);
@@ -74,7 +75,7 @@ template <int PREC>
 __device__ __forceinline__ cplx<typename Prec<PREC>::real> load_comp(const typename Prec<PREC>::vec* f, int comp, int cb,
                                                                      int Vh) {
   if constexpr (PREC == PFMP_F32) {
-    const float2 w = __ldg(reinterpret_cast<const float2*>(f + (size_t)(comp >> 1) * Vh + cb) + (comp & 1));
+    const float2 w = ld_live(reinterpret_cast<const float2*>(f + (size_t)(comp >> 1) * Vh + cb) + (comp & 1));
     return mk(w.x, w.y);
   } else if constexpr (PREC == PREC_DF) {
     return c_of(__ldg(f + (size_t)comp * Vh + cb));

@@ -45,9 +45,9 @@ void spinor_unpack_any(pfmp_ctx* c, double* dst, int where, const void* src, int
 void spinor_pack_any(pfmp_ctx* c, void* dst, int prec, const double* src, int where, int parity);
 
 // ------------------------------------------------------------------ kernels
-__global__ void k_mom_update(double* __restrict__ p, const double* __restrict__ F, double eps, long n) {
+__global__ void k_mom_update(double* p, const double* F, double eps, long n) {
   chain_enter();
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) p[i] -= eps * F[i];
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) p[i] = ld_live(p + i) - eps * ld_live(F + i);
 }
 
 __global__ void k_sumsq(const double* __restrict__ p, long n, ReduceBuf rb, double* out) {
@@ -58,17 +58,20 @@ __global__ void k_sumsq(const double* __restrict__ p, long n, ReduceBuf rb, doub
 }
 
 // U <- exp(i eps P) U, P = sum_a p_a T_a, then reunitarise (FP64 master field)
-__global__ void k_link_update(double2* U, const double* __restrict__ mom, Geom g, double eps) {
+__global__ void k_link_update(double2* U, const double* mom, Geom g, double eps) {
   chain_enter();
   const int cb = blockIdx.x * blockDim.x + threadIdx.x;
   const int pm = blockIdx.y;  // parity * 4 + mu
   if (cb >= g.Vh) return;
   double c[8];
-  for (int a = 0; a < 8; ++a) c[a] = mom[(size_t)(pm * 8 + a) * g.Vh + cb];
+  for (int a = 0; a < 8; ++a) c[a] = ld_live(mom + (size_t)(pm * 8 + a) * g.Vh + cb);
   Mat3<double> E = expm_algebra(c, eps);
   Mat3<double> L;
   double2* base = U + (size_t)(pm * 9) * g.Vh;
-  load_link18(L, base, cb, g.Vh);
+  for (int k = 0; k < 9; ++k) {
+    const double2 v = ld_live(base + (size_t)k * g.Vh + cb);
+    L.m[k / 3][k % 3] = mk(v.x, v.y);
+  }
   Mat3<double> N = matmul(E, L);
   reunitarise(N);
   store_link18(base, N, cb, g.Vh);
@@ -105,7 +108,7 @@ static int grid_for(long n) {
 // links (deterministic grid sum), *maxbits = max over links (the bit patterns of
 // non-negative doubles order like the values, so an integer atomicMax is exact and
 // independent of scheduling); *maxbits must be zero on entry
-__global__ void k_force_norm(const double* __restrict__ F, int Vh, ReduceBuf rb, double* out,
+__global__ void k_force_norm(const double* F, int Vh, ReduceBuf rb, double* out,
                              unsigned long long* maxbits) {
   chain_enter();
   double v[1] = {0.0};
@@ -116,7 +119,7 @@ __global__ void k_force_norm(const double* __restrict__ F, int Vh, ReduceBuf rb,
     double s = 0.0;
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
-      const double f = F[(size_t)(pm * 8 + a) * Vh + cb];
+      const double f = ld_live(F + (size_t)(pm * 8 + a) * Vh + cb);
       s += f * f;
     }
     const double n = sqrt(s);

@@ -124,7 +124,7 @@ __device__ __forceinline__ float4 xpby_real(float4 r, double bd, float4 p) {
 // every shift in turn cost 10-25 us an iteration, FP64 divisions in a serial chain: the
 // kernel at 24^3x48 with 13 shifts 41 -> 27 us.)
 template <typename V>
-__global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V* __restrict__ Ap, long n, ReduceBuf rb,
+__global__ void k_ms_r(V* __restrict__ r, const V* r_prev, const V* Ap, long n, ReduceBuf rb,
                        CGScalars* s, MSSeed* sd, MSShift* sh, int ns, int* act, int slot, bool chained) {
   chain_enter(chained);
   if (s->done) {  // a block that starts after the end has no iterations
@@ -134,7 +134,7 @@ __global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V*
   const double al = s->alpha;
   typename NormOf<V>::type acc;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const V rr = sub_real(r_prev[i], al, Ap[i]);
+    const V rr = sub_real(ld_live(r_prev + i), al, ld_live(Ap + i));
     r[i] = rr;
     acc.add(rr);
   }
@@ -195,12 +195,12 @@ __global__ void k_ms_r(V* __restrict__ r, const V* __restrict__ r_prev, const V*
 
 // seed direction p = r + beta p
 template <typename V>
-__global__ void k_ms_p(V* __restrict__ p, const V* __restrict__ r, long n, const CGScalars* s, bool chained) {
+__global__ void k_ms_p(V* p, const V* r, long n, const CGScalars* s, bool chained) {
   chain_enter(chained);
   if (s->done) return;
   const double be = s->beta;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    p[i] = xpby_real(r[i], be, p[i]);
+    p[i] = xpby_real(ld_live(r + i), be, ld_live(p + i));
 }
 
 // coefficients and fields of one shift in the arithmetic of its vectors
@@ -239,8 +239,8 @@ struct MSRing {
   V* r[kMsBlock];
 };
 template <typename V>
-__global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRing<V> ring, const MSShift* __restrict__ sh,
-                                                  const int* __restrict__ act, const MSSeed* sd, long n, bool chained) {
+__global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRing<V> ring, const MSShift* sh,
+                                                  const int* act, const MSSeed* sd, long n, bool chained) {
   chain_enter(chained);
   using C = typename MSCoef<V>::C;
   const int cnt = sd->count;
@@ -271,10 +271,10 @@ __global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRi
       V rr[kMsBlock];
 #pragma unroll
       for (int b = 0; b < kMsBlock; ++b)
-        if (b < cnt) rr[b] = ring.r[b][i];
+        if (b < cnt) rr[b] = ld_live(ring.r[b] + i);
 #pragma unroll 2
       for (int j = 0; j < m; ++j) {
-        V pk = sp[j][i], xk = sx[j][i];
+        V pk = ld_live(sp[j] + i), xk = ld_live(sx[j] + i);
         int last = 0;
 #pragma unroll
         for (int b = 0; b < kMsBlock; ++b) {
@@ -295,12 +295,14 @@ __global__ void __launch_bounds__(kBlock) k_ms_xp(V* const* x, V* const* p, MSRi
 // y = a x + b y (complex a, b) on FP64 or FP32 even fields; with b = 0, y = a x without
 // reading y (its previous contents may be anything, NaN included)
 template <typename V>
-__global__ void k_caxpby(double2 a, const V* __restrict__ x, double2 b, V* __restrict__ y, long n) {
+__global__ void k_caxpby(double2 a, const V* x, double2 b, V* y, long n) {
   chain_enter();
   const bool read_y = b.x != 0.0 || b.y != 0.0;
   const double2 zero = make_double2(0.0, 0.0);
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    y[i] = read_y ? axpby_c(a, x[i], b, y[i]) : axpby_c(a, x[i], zero, x[i]);
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    const V xi = ld_live(x + i);
+    y[i] = read_y ? axpby_c(a, xi, b, ld_live(y + i)) : axpby_c(a, xi, zero, xi);
+  }
 }
 
 static int ms_grid(long n) {

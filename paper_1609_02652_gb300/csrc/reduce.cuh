@@ -10,9 +10,12 @@ namespace pfmp {
 // launched with launch_chained may become resident while its predecessor drains, and
 // chain_enter, its first statement, waits until the predecessor has completed (its writes
 // are then visible) after letting its own successor come up in the same way.  A successor
-// launched in the ordinary way waits for completion as always.  In a kernel that takes
-// chain_enter, loads through the read-only path come after a branch or inside a loop: in the
-// entry block the compiler could move them above the wait.
+// launched in the ordinary way waits for completion as always.  Such a kernel is resident
+// while its predecessor still writes, so it must not read what a predecessor writes through
+// the read-only path (__ldg, const __restrict__ parameters: data that stay the same for as
+// long as the kernel lives, which the compiler may also load above the wait): it takes ld_live,
+// or plain loads of pointers without those qualifiers.  The links and clover blocks of an
+// operator are exempt: clover_build waits for the stream before any kernel may use them.
 // K at 4^3x8 (four launches of k_hop_pair) 16.4 -> 10.7 us.  The FP64 stencils and force
 // contractions gain nothing (the FP64 force at 6x10x14x18 +2%), nor do the one-thread-per-site
 // stencils (K at 32^3x64 +2%): those are launched in the ordinary way.  Inside a CUDA graph
@@ -25,6 +28,33 @@ __device__ __forceinline__ void chain_enter() {
 }
 __device__ __forceinline__ void chain_enter(bool chained) {
   if (chained) chain_enter();
+}
+// An ordinary coherent load, written so that it stays below chain_enter (volatile assembly keeps
+// its order) without holding back the loads after it.
+__device__ __forceinline__ float ld_live(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ld_live(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_live(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_live(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_live(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
 }
 // whether launches on st are chained
 inline bool chain_launches(cudaStream_t st) {

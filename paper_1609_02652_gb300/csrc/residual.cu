@@ -11,18 +11,18 @@
 
 namespace pfmp {
 
-__global__ void k_split_df(const double2* __restrict__ x, float4* __restrict__ y, long n) {
+__global__ void k_split_df(const double2* x, float4* __restrict__ y, long n) {
   chain_enter();
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) y[i] = split2(x[i]);
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) y[i] = split2(ld_live(x + i));
 }
 
-__global__ void k_residual_df(const double2* __restrict__ b, const float4* __restrict__ kx, double2* __restrict__ r,
+__global__ void k_residual_df(const double2* b, const float4* kx, double2* __restrict__ r,
                               long n, ReduceBuf rb, double* out) {
   chain_enter();
   double v[1] = {0.0};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const double2 bb = b[i];
-    const float4 k = kx[i];
+    const double2 bb = ld_live(b + i);
+    const float4 k = ld_live(kx + i);
     const double2 d = make_double2(bb.x - ((double)k.x + (double)k.y), bb.y - ((double)k.z + (double)k.w));
     r[i] = d;
     v[0] += d.x * d.x + d.y * d.y;
@@ -37,11 +37,11 @@ static int rgrid(long n) {
 }
 
 // r = b - r, |r|^2 -> *out
-__global__ void k_b_minus_r(const double2* __restrict__ b, double2* __restrict__ r, long n, ReduceBuf rb, double* out) {
+__global__ void k_b_minus_r(const double2* b, double2* r, long n, ReduceBuf rb, double* out) {
   chain_enter();
   double v[1] = {0.0};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const double2 bb = b[i], kx = r[i];
+    const double2 bb = ld_live(b + i), kx = ld_live(r + i);
     const double2 d = make_double2(bb.x - kx.x, bb.y - kx.y);
     r[i] = d;
     v[0] += d.x * d.x + d.y * d.y;
