@@ -369,7 +369,14 @@ typedef struct {
 #define PFMP_SCHEME_1PF2MP 6
 int pfmp_action_scheme(int scheme, int p1, int p2, pfmp_action_def* def);
 /* PFMP_E_INVALID for out-of-range kinds, kappa indices or counts; PFMP_E_UNSUPPORTED for
- * odd filter orders or orders that do not factorise.                                    */
+ * odd filter orders or orders that do not factorise.
+ * Device memory is taken when a force first needs it and kept by the action: for a filter
+ * of m roots m half-lattice fields and 40 for the contractions, and, only where there is
+ * room, three more per root that save their recomputation (at most a sixteenth of the
+ * device's memory and a quarter of what is free then; the result does not depend on it).
+ * A clover force keeps 1728 bytes per lattice site (FP64; FP32 half of it) on the
+ * context, a multi-shift solve eight fields of its precision and one FP64 field per shift
+ * on the operator.                                                                       */
 int pfmp_action_create_def(pfmp_ctx* ctx, const pfmp_action_def* def, pfmp_action** action);
 int pfmp_action_create(pfmp_ctx* ctx, const pfmp_action_params* prm, pfmp_action** action);
 int pfmp_action_destroy(pfmp_action* action);

@@ -114,6 +114,7 @@ inline size_t spinor_bytes(const Geom& g, int prec) {
   return (size_t)g.Vh * 24 * (prec == PFMP_F64 ? 8 : 4);
 }
 void* dev_alloc(size_t bytes);
+void* dev_try_alloc(size_t bytes);
 void dev_free(void* p);
 
 // core.cu

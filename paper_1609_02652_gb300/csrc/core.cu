@@ -19,6 +19,17 @@ long long launch_count() { return g_launches.load(); }
 void set_last_error(const std::string& s) { g_last_error = s; }
 const char* last_error() { return g_last_error.c_str(); }
 
+// null when the device has no room for it (any other error throws)
+void* dev_try_alloc(size_t bytes) {
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  PFMP_CUDA(e);
+  return p;
+}
 void* dev_alloc(size_t bytes) {
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);

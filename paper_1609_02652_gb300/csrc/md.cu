@@ -32,6 +32,7 @@
 
 #include "context.h"
 #include "fields.cuh"
+#include "image_pool.h"
 #include "su3.cuh"
 
 using cd = std::complex<double>;
@@ -165,13 +166,14 @@ struct pfmp_action {
   double* mom = nullptr;  // [2][4][8][Vh]
   double2* U0 = nullptr;  // saved master gauge field
   std::vector<double2*> ev;  // even FP64 temporaries
-  std::vector<double2*> xs;  // multi-shift solutions
+  std::vector<double2*> xs;  // multi-shift solutions, filter chains
   // FP32 force path (force_prec = PFMP_F32): even temporaries, solutions and filter
   // chains
   std::vector<float4*> ev32;
   std::vector<float4*> xs32;
   // half-lattice scratch of the batched force contractions, FP64 [0] and FP32 [1]
   std::vector<void*> fbuf[2];
+  ImagePool images[2];  // the images of a filter force's chain, FP64 and FP32
   int force_evals = 0;
 };
 
@@ -214,17 +216,21 @@ void cg_tol(pfmp_action* A, pfmp_op* op, void* x, const void* b, double tol) {
 }
 void cg64(pfmp_action* A, pfmp_op* op, void* x, const void* b) { cg_tol(A, op, x, b, A->def.tol); }
 
+// even field k of A->xs (FP64) or A->xs32 (FP32)
+void* solution(pfmp_action* A, int prec, int k) {
+  if (prec == PFMP_F64) {
+    while ((int)A->xs.size() <= k) A->xs.push_back((double2*)dev_alloc(spb(A)));
+    return A->xs[k];
+  }
+  while ((int)A->xs32.size() <= k) A->xs32.push_back((float4*)dev_alloc(spinor_bytes(A->ctx->g, PFMP_F32)));
+  return A->xs32[k];
+}
+
 // multi-shift solutions into A->xs (FP64, at the action's tolerance) or A->xs32 (FP32,
 // at the MD tolerance: the solves of the FP32 forces)
 void multishift(pfmp_action* A, pfmp_op* op, const std::vector<cd>& sig, const void* b, int prec = PFMP_F64) {
   std::vector<void*> x(sig.size());
-  if (prec == PFMP_F64) {
-    while (A->xs.size() < sig.size()) A->xs.push_back((double2*)dev_alloc(spb(A)));
-    for (size_t k = 0; k < sig.size(); ++k) x[k] = A->xs[k];
-  } else {
-    while (A->xs32.size() < sig.size()) A->xs32.push_back((float4*)dev_alloc(spinor_bytes(A->ctx->g, PFMP_F32)));
-    for (size_t k = 0; k < sig.size(); ++k) x[k] = A->xs32[k];
-  }
+  for (size_t k = 0; k < sig.size(); ++k) x[k] = solution(A, prec, (int)k);
   int it;
   double res;
   long kap;
@@ -235,15 +241,11 @@ void multishift(pfmp_action* A, pfmp_op* op, const std::vector<cd>& sig, const v
 }
 
 // half-lattice scratch field i of the fermion forces in precision prec, kept by the action
-void*& fslot(pfmp_action* A, int prec, int i) {
+void* fscratch(pfmp_action* A, int prec, int i) {
   auto& v = A->fbuf[prec == PFMP_F64 ? 0 : 1];
   if ((int)v.size() <= i) v.resize(i + 1, nullptr);
+  if (!v[i]) v[i] = dev_alloc(spinor_bytes(A->ctx->g, prec));
   return v[i];
-}
-void* fscratch(pfmp_action* A, int prec, int i) {
-  void*& p = fslot(A, prec, i);
-  if (!p) p = dev_alloc(spinor_bytes(A->ctx->g, prec));
-  return p;
 }
 
 // An even field v and what the contractions need of it, all of them on the way to K v:
@@ -262,7 +264,6 @@ struct Images {
 // them being written ahead of its use.
 struct ForceBatch {
   static constexpr int kRing = kMaxDerivSets / 2 + 1;
-  static constexpr int kChain = 8 * kRing;  // scratch index of the chains' fields
   pfmp_action* A;
   int prec;
   DerivBatch b;
@@ -405,6 +406,8 @@ void action_destroy(pfmp_action* A) {
   for (auto p : A->xs32) dev_free(p);
   for (auto& v : A->fbuf)
     for (auto p : v) dev_free(p);
+  for (auto& v : A->images)
+    for (auto p : v.f) dev_free(p);
   for (auto op : A->ops) op_delete(op);
   delete A;
 }
@@ -593,38 +596,30 @@ void action_eval(pfmp_action* A, double* S) {
 // with a root of each conjugate pair in R would halve that again, with chains that start
 // from each other; its FP32 force is up to 1.9 times further from the FP64 one at order 64.)
 // MD at 24^3x48 with filters of order 12 and 64, this and the correction force below: 825 ->
-// 600 ms, a 4^4 trajectory 43 -> 38 ms.  The images of chi_k are kept (four half-lattice fields per root) while that takes at most half
-// of the free device memory, and recomputed when eta_k is there otherwise (three stencils
-// more).
+// 600 ms, a 4^4 trajectory 43 -> 38 ms.  The images of chi_k are kept where they fit (ImagePool:
+// three half-lattice fields per root), and recomputed when eta_k is there otherwise (three
+// stencils more per root: the FP32 force of order 64 at 24^3x48 takes 47.7 ms with all images
+// kept, 57.8 with five).
 static void force_filter(pfmp_action* A, Term& T, pfmp_op* W, int prec, const void* phi) {
   pfmp_ctx* c = A->ctx;
   const int m = (int)T.q.size();
   ForceBatch fb(A, prec);
-  const int base = ForceBatch::kChain;
-  bool keep = fslot(A, prec, base + 4 * m - 1) != nullptr;
-  if (!keep) {
-    size_t free_b = 0, total_b = 0;
-    PFMP_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    keep = 4.0 * m * spinor_bytes(c->g, prec) <= 0.5 * (double)free_b;
-  }
-  // chi_k, and with `keep` its images
-  auto chi = [&](int k) { return fb.field(base + (keep ? 4 * k : k)); };
-  auto kept = [&](int k) {
-    const int i = base + 4 * k;
-    return Images{chi(k), fb.field(i + 1), fb.field(i + 2), fb.field(i + 3)};
-  };
-  caxpby(c, prec, T.c, phi, 0.0, chi(m - 1));
-  for (int k = m - 1; k >= 0; --k) {
-    if (k == 0) {
-      if (keep) images(W, prec, kept(k));
-      break;
-    }
-    if (keep)
-      kop_images(W, prec, chi(k - 1), kept(k));
+  std::vector<void*> chi(m);
+  for (int k = 0; k < m; ++k) chi[k] = solution(A, prec, k);
+  for (int i = 0; i < 8 * ForceBatch::kRing; ++i) fb.field(i);  // what the force needs comes before what it may keep
+  ImagePool& pool = A->images[prec == PFMP_F64 ? 0 : 1];
+  const int keep = pool.reserve(
+      m, spinor_bytes(c->g, prec), [](size_t* f, size_t* t) { PFMP_CUDA(cudaMemGetInfo(f, t)); }, dev_try_alloc, dev_free);
+  auto kept = [&](int k) { return Images{chi[k], pool.field(k, 0), pool.field(k, 1), pool.field(k, 2)}; };
+  caxpby(c, prec, T.c, phi, 0.0, chi[m - 1]);
+  for (int k = m - 1; k > 0; --k) {
+    if (k < keep)
+      kop_images(W, prec, chi[k - 1], kept(k));
     else
-      kop(W, prec, chi(k - 1), chi(k), nullptr, nullptr);
-    caxpby(c, prec, -T.q[k], chi(k), 1.0, chi(k - 1));
+      kop(W, prec, chi[k - 1], chi[k], nullptr, nullptr);
+    caxpby(c, prec, -T.q[k], chi[k], 1.0, chi[k - 1]);
   }
+  if (keep > 0) images(W, prec, kept(0));
   for (int k = 0; k < m; ++k) {
     const Images eta = fb.ring_images(k == 0 ? phi : fb.ring(k), k);
     if (k + 1 < m) {
@@ -635,10 +630,10 @@ static void force_filter(pfmp_action* A, Term& T, pfmp_op* W, int prec, const vo
       images(W, prec, eta);
     }
     Images x;
-    if (keep) {
+    if (k < keep) {
       x = kept(k);
     } else {
-      x = fb.ring_images(chi(k), k, 1);
+      x = fb.ring_images(chi[k], k, 1);
       images(W, prec, x);
     }
     fb.add_K(W, eta, x, 1.0);
@@ -714,7 +709,7 @@ static void fermion_force(pfmp_action* A, Term& T, pfmp_op* W, const void* phi) 
   } else if (T.d.kind == PFMP_KIND_FILTERCORR) {
     multishift(A, W, T.sig, in_prec(phi, 0), prec);
     std::vector<const void*> x;
-    for (size_t k = 0; k < T.sig.size(); ++k) x.push_back(f32 ? (const void*)A->xs32[k] : (const void*)A->xs[k]);
+    for (size_t k = 0; k < T.sig.size(); ++k) x.push_back(solution(A, prec, (int)k));
     force_filtercorr(A, T, W, prec, x);
   } else if (T.d.kind == PFMP_KIND_RATIO) {
     pfmp_op* Mb = A->ops[T.d.b];
