@@ -588,14 +588,16 @@ __device__ __forceinline__ double spinor_norm2(const Spinor<T>& v) {
     for (int c = 0; c < 3; ++c) t += (double)norm2(v.s[s][c]);
   return t;
 }
-// FP32: the site's twelve terms as a pair sum, as exact as in FP64 without its pipe
+// FP32: the site's twelve terms without the FP64 pipe (TripleSum), or in FP64 where their sum
+// is beyond FP32
 __device__ __forceinline__ double spinor_norm2(const Spinor<float>& v) {
-  PairSum t;
+  TripleSum t;
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
     for (int c = 0; c < 3; ++c) t.add(norm2(v.s[s][c]));
-  return t.value();
+  if (t.ok()) return t.value();
+  return spinor_norm2<float>(v);
 }
 
 }  // namespace pfmp

@@ -88,18 +88,21 @@ __device__ __forceinline__ float4 sub_real(float4 r, double ad, float4 q) {
   return make_float4(r.x - a * q.x, r.y - a * q.y, r.z - a * q.z, r.w - a * q.w);
 }
 __device__ __forceinline__ double nrm(double2 v) { return v.x * v.x + v.y * v.y; }
+__device__ __forceinline__ double nrm(float4 v) { return (double)(v.x * v.x + v.y * v.y) + (double)(v.z * v.z + v.w * v.w); }
 // |v|^2 added to a thread's running sum
 struct NormSum64 {
   double t = 0.0;
   __device__ __forceinline__ void add(double2 v) { t += nrm(v); }
+  __device__ __forceinline__ bool ok() const { return true; }
   __device__ __forceinline__ double value() const { return t; }
 };
 struct NormSum32 {
-  PairSum t;
+  TripleSum t;
   __device__ __forceinline__ void add(float4 v) {
     t.add(v.x * v.x + v.y * v.y);
     t.add(v.z * v.z + v.w * v.w);
   }
+  __device__ __forceinline__ bool ok() const { return t.ok(); }
   __device__ __forceinline__ double value() const { return t.value(); }
 };
 template <typename V>
@@ -139,6 +142,10 @@ __global__ void k_ms_r(V* __restrict__ r, const V* r_prev, const V* Ap, long n, 
     acc.add(rr);
   }
   double v[1] = {acc.value()};
+  if (!acc.ok()) {
+    v[0] = 0.0;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) v[0] += nrm(r[i]);
+  }
   double t[1];
   if (!grid_sum_last<1>(v, rb, t)) return;
   __shared__ int wcount[kBlock / 32];

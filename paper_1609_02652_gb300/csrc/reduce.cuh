@@ -83,18 +83,27 @@ struct ReduceBuf {
 constexpr int kMaxSums = 4;
 constexpr int kMaxReduceBlocks = 65536;
 
-// A thread's sum of FP32 values as an unevaluated pair hi + lo (Knuth's TwoSum), ~48 bits,
-// turned into FP64 once: an FP64 add and a conversion per value cost 16 cycles of the SM's
-// FP64 pipe per warp each (22 us of a 77 us stencil with a norm at 24^3x48), TwoSum's seven
-// FP32 operations a quarter of a cycle each.
-struct PairSum {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-    hi = s;
+// A thread's sum of FP32 values without the FP64 pipe, turned into FP64 once: an FP64 add and
+// a conversion per value cost 16 cycles of the SM's FP64 pipe per warp each (22 us of a 77 us
+// stencil with a norm at 24^3x48), thirteen FP32 operations under half a cycle each.  The sum is an
+// unevaluated hi + mid + lo: Knuth's TwoSum adds the value to hi and the error of that to mid,
+// and only the error of the second sum is rounded when it is added to lo, a 2^-72 of the
+// running sum.  So value() is the sum of the values rounded to FP64 about once, where FP64
+// additions in turn round at each (a pair hi + lo would stop at 2^-48).  ok() is false when the
+// sum left the range of FP32 or a value was not finite: the caller then adds in FP64.
+struct TripleSum {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
+  // a + b = s + the return value exactly
+  static __device__ __forceinline__ float two_sum(float a, float b, float& s) {
+    s = __fadd_rn(a, b);
+    const float c = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, c)), __fsub_rn(b, c));
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ void add(float v) {
+    lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, v, hi), mid));
+  }
+  __device__ __forceinline__ bool ok() const { return fabsf(hi) < 3e38f; }
+  __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
 
 template <int N>
