@@ -55,6 +55,7 @@ struct MSSeed {
   double alpha_prev, beta_prev;
   int nact;        // shifts active in the block's first iteration, listed in act[]
   int count;       // iterations of the block that ran
+  int ns;          // shifts of this solve
 };
 
 __device__ __forceinline__ double2 cm(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
@@ -128,7 +129,7 @@ __device__ __forceinline__ float4 xpby_real(float4 r, double bd, float4 p) {
 // kernel at 24^3x48 with 13 shifts 41 -> 27 us.)
 template <typename V>
 __global__ void k_ms_r(V* __restrict__ r, const V* r_prev, const V* Ap, long n, ReduceBuf rb,
-                       CGScalars* s, MSSeed* sd, MSShift* sh, int ns, int* act, int slot, bool chained) {
+                       CGScalars* s, MSSeed* sd, MSShift* sh, int* act, int slot, bool chained) {
   chain_enter(chained);
   if (s->done) {  // a block that starts after the end has no iterations
     if (slot == 0 && blockIdx.x == 0 && threadIdx.x == 0) sd->count = 0;
@@ -151,6 +152,7 @@ __global__ void k_ms_r(V* __restrict__ r, const V* r_prev, const V* Ap, long n, 
   __shared__ int wcount[kBlock / 32];
   const double rr0 = s->rr, stop = s->stop_rr, beta = t[0] / rr0;
   const double ap = sd->alpha_prev, bp = sd->beta_prev;
+  const int ns = sd->ns;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int any = 0, listed = 0;
   for (int k0 = 0; k0 < ns; k0 += blockDim.x) {
@@ -386,19 +388,21 @@ void ms_work_free(pfmp_op* op) {
 }
 
 template <typename V>
-static void ms_chunk(pfmp_op* op, int prec, MSWork& w, int ns, void* pseed, void* Ap, long n, int chunk) {
+static void ms_chunk(pfmp_op* op, int prec, MSWork& w, void* pseed, void* Ap, long n, int chunk) {
   pfmp_ctx* c = op->ctx;
   const bool chained = chain_launches(c->stream);
   MSRing<V> ring;
   for (int b = 0; b < kMsBlock; ++b) ring.r[b] = (V*)w.ring[prec == PFMP_F64 ? 0 : 1][b];
-  // rows of shifts until the pass has about four blocks per SM
-  const int nb = ms_grid(n), rows = std::max(1, std::min(ns, 152 * 4 / nb));
+  // rows of shifts until the pass has about four blocks per SM; for as many shifts as the
+  // workspace holds, so that a chunk serves solves with any number of them (the rows beyond
+  // this solve's shifts end at once)
+  const int nb = ms_grid(n), rows = std::max(1, std::min(w.cap, 152 * 4 / nb));
   for (int k = 0; k < chunk; ++k) {
     const int slot = k % kMsBlock;
     kop(op, prec, Ap, pseed, &op->scal->pAp, op->scal);
     // the residual before a chunk is in the last slot (every chunk but the last is whole blocks)
     const V* prev = ring.r[slot == 0 ? kMsBlock - 1 : slot - 1];
-    launch_chained(k_ms_r<V>, nb, kBlock, c->stream, ring.r[slot], prev, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh, ns,
+    launch_chained(k_ms_r<V>, nb, kBlock, c->stream, ring.r[slot], prev, (const V*)Ap, n, c->rb, op->scal, w.d_seed, w.d_sh,
                                             w.d_act, slot, chained);
     PFMP_CHECK_LAUNCH();
     launch_chained(k_ms_p<V>, nb, kBlock, c->stream, (V*)pseed, ring.r[slot], n, op->scal, chained);
@@ -412,7 +416,10 @@ static void ms_chunk(pfmp_op* op, int prec, MSWork& w, int ns, void* pseed, void
 }
 
 // Up to this many sites per parity the kernels of an iteration are shorter than the
-// host takes to launch them, and a chunk is replayed as a CUDA graph (as the CG's).
+// host takes to launch them, and a chunk is replayed as a CUDA graph (as the CG's).  The graph
+// depends on the workspace only, not on the solve's shifts: solves that alternate between
+// numbers of shifts share it (with a capture for each change of their number a solve of 0.21 ms
+// took 0.35).  A chunk cut short by the iteration cap is launched directly.
 constexpr int kMsGraphMax = 32768;
 
 // x[k] = (K + sigma_k)^{-1} b in FP64 or FP32 (x, b of precision prec).  Returns the
@@ -470,7 +477,7 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
   PFMP_CUDA(cudaMemcpyAsync(w.d_p, hp.data(), ns * sizeof(void*), cudaMemcpyHostToDevice, c->stream));
   PFMP_CUDA(cudaMemcpyAsync(w.d_sh, hs.data(), ns * sizeof(MSShift), cudaMemcpyHostToDevice, c->stream));
   PFMP_CUDA(cudaMemcpyAsync(w.d_act, act.data(), ns * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  MSSeed sd{1.0, 0.0, ns, 0};
+  MSSeed sd{1.0, 0.0, ns, 0, ns};
   PFMP_CUDA(cudaMemcpyAsync(w.d_seed, &sd, sizeof(MSSeed), cudaMemcpyHostToDevice, c->stream));
   CGScalars* h = op->h_scal;
   *h = CGScalars{};
@@ -483,12 +490,12 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
     const int chunk = check < max_iter - done ? check : max_iter - done;
     auto launch = [&]() {
       if (prec == PFMP_F64)
-        ms_chunk<double2>(op, prec, w, ns, pseed, Ap, n, chunk);
+        ms_chunk<double2>(op, prec, w, pseed, Ap, n, chunk);
       else
-        ms_chunk<float4>(op, prec, w, ns, pseed, Ap, n, chunk);
+        ms_chunk<float4>(op, prec, w, pseed, Ap, n, chunk);
     };
-    if (c->g.Vh <= kMsGraphMax && !c->prof.on) {
-      const void* key[4] = {w.d_sh, w.d_x, w.d_p, (const void*)(intptr_t)ns};
+    if (c->g.Vh <= kMsGraphMax && !c->prof.on && chunk == check) {
+      const void* key[4] = {w.d_sh, w.d_x, w.d_p, w.d_act};
       run_graph(op, op->graph[prec == PFMP_F64 ? kGraphMs64 : kGraphMs32], key, chunk, launch);
     } else {
       launch();
