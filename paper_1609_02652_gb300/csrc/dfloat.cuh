@@ -10,12 +10,14 @@
 // Addition is the "sloppy" df add (TwoSum of the high parts, low parts added, one
 // renormalisation): its error is bounded by a few df ulps of |x| + |y|, which is what a
 // stencil sum of many terms needs.  Multiplication is TwoProd of the high parts plus the
-// cross terms.  Products and the running sums of multiply-adds are not renormalised: the low
-// part of such a sum holds the rounding errors of its few terms, some 2^-24 of the largest
-// partial result, and is itself rounded at 2^-48 of that, as a renormalised one would be.
-// 12 FP32 instructions per multiply-add (18 with two renormalisations).  GB300, r = b - K x with
-// its copies, before / now: 16^3x32 372 / 283 us, 32^3x64 4310 / 3312 us; |r_df - r_f64| / |K x|
-// at 32^3x64 4.8e-15 / 4.3e-15.
+// cross terms, not renormalised: a product's low part is within a few 2^-24 of its high part, and
+// the sums that take it renormalise.  A multiply-add is 15 FP32 instructions (18 with its product
+// renormalised, 12 without either).  Without the sums' renormalisation too, low parts grow along a
+// row of products and so do their roundings: |r_df - r_f64| / |K x| of Gaussian x at 16^3x32 was
+// 4.3e-15 with c_sw = 1 and 2.5e-15 without a clover term; it is 3.9e-15 and 2.1e-15 now, 4.8e-15
+// and 2.1e-15 with both renormalised (on smooth x 1.10e-14 now, 1.23e-14 with both).  GB300,
+// r = b - K x with its copies, both / now / neither: 16^3x32 372 / 298 / 283 us, 32^3x64
+// 4310 / 3550 / 3340 us.
 #pragma once
 #include "fields.cuh"
 #include "mad.cuh"
@@ -63,7 +65,7 @@ __device__ __forceinline__ df operator*(df x, df y) {
 
 __device__ __forceinline__ df mad(df x, df y, df z) {
   const df p = x * y, s = df_two_sum(z.hi, p.hi);
-  return df(s.hi, __fadd_rn(z.lo, __fadd_rn(s.lo, p.lo)));
+  return df_fast_two_sum(s.hi, __fadd_rn(__fadd_rn(z.lo, p.lo), s.lo));
 }
 
 template <>
@@ -77,7 +79,7 @@ struct Prec<2> {  // double-float, used only inside the library (the true residu
 constexpr int PREC_DF = 2;
 
 __device__ __forceinline__ cplx<df> c_of(float4 v) { return mk(df(v.x, v.y), df(v.z, v.w)); }
-__device__ __forceinline__ float4 v_of(cplx<df> c) {
+__device__ __forceinline__ float4 v_of(cplx<df> c) {  // renormalised: c may be a product
   const df re = df_fast_two_sum(c.re.hi, c.re.lo), im = df_fast_two_sum(c.im.hi, c.im.lo);
   return make_float4(re.hi, re.lo, im.hi, im.lo);
 }
