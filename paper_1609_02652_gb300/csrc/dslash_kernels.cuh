@@ -115,8 +115,10 @@ void launch_site(const HopParams<PREC>& a, int bs, cudaStream_t st) {
     const long slots = 152L * m * 128 / bs;
     n = nblocks(n, (int)((n + slots - 1) / slots));
   }
+  // FP16 storage without a sum needs 127 registers, whether it may have 255 or 128
+  constexpr int B2 = PREC == PFMP_F32 || RED ? 2 : 4;
   switch (m) {
-    case 2: k_hop<PREC, DAG, EPI, RED, 2><<<n, bs, 0, st>>>(a); break;
+    case 2: k_hop<PREC, DAG, EPI, RED, B2><<<n, bs, 0, st>>>(a); break;
     case 4: k_hop<PREC, DAG, EPI, RED, 4><<<n, bs, 0, st>>>(a); break;
     default: k_hop<PREC, DAG, EPI, RED, B><<<n, bs, 0, st>>>(a);
   }

@@ -212,16 +212,6 @@ __device__ __forceinline__ void load_clover(HermBlock<double> b[2], const double
   load_clover_block(b[0], f, 0, cb, Vh);
   load_clover_block(b[1], f, 1, cb, Vh);
 }
-__device__ __forceinline__ void store_clover(double2* __restrict__ f, const HermBlock<double> b[2], int cb, int Vh) {
-#pragma unroll
-  for (int blk = 0; blk < 2; ++blk) {
-    double2* g = f + (size_t)(18 * blk) * Vh;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) g[(size_t)k * Vh + cb] = make_double2(b[blk].d[2 * k], b[blk].d[2 * k + 1]);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) g[(size_t)(3 + k) * Vh + cb] = make_double2(b[blk].o[k].re, b[blk].o[k].im);
-  }
-}
 __device__ __forceinline__ void load_clover(HermBlock<float> b[2], const float4* __restrict__ f, int cb, int Vh) {
 #pragma unroll
   for (int blk = 0; blk < 2; ++blk) {

@@ -35,7 +35,7 @@ struct HopParams {
 // Register bound (resident 128-thread blocks per SM) of the one-thread-per-site FP32 and FP16
 // stencils for Vh sites, `most` where the lattice fills the SMs many times.  A thread has 90
 // 16-byte loads to make; the fewer blocks an SM gets, the more registers it can spare to keep
-// them in flight (255 at 2, 128 at 4, 72 at 7).  4 is taken where its whole waves of blocks
+// them in flight (196 at 2, 252 with a sum; 128 at 4, 72 at 7).  4 is taken where its whole waves of blocks
 // cover the lattice with a tenth fewer slots.  GB300, FP32, us per K with a bound of 7 / 4 / 2:
 // 16^4 (1.7 blocks per SM) 37.0 / 32.9 / 29.8, 16^3x24 (2.5) 41.0 / 36.9 / 41.1, 16^3x32 (3.4)
 // 50.6 / 43.9 / 49.2, 18^3x36 (5.4) 80 / 88 / 85, 16^2x24x48 (7.6) 130 / 108 / 118, 24^3x48 (17)

@@ -406,13 +406,13 @@ __global__ void __launch_bounds__(8 * kPairSites, 5) k_hop_pair(HopParams<PREC> 
 // Several threads per site below, one thread per site from these sizes on (sites per
 // parity; us per K of four launches, GB300):
 //  * FP32: a lattice with few sites leaves k_hop's 128-site blocks on a few SMs, each waiting
-//    for one thread's chain of eight neighbours.  k_hop_pair against k_hop (255 registers):
+//    for one thread's chain of eight neighbours.  k_hop_pair against k_hop (196 registers):
 //    16.5 / 24.7 at 256 to 2048, 17.2 / 24.7 at 4096, 24.7 / 24.6 at 6144, 32.9 / 24.6 at 20736,
 //    41.0 / 28.8 at 27648.
 //  * FP64 and double-float, always several threads: k_hop_tile (8-site blocks, 16 threads
 //    per site) while the 16-site blocks of k_hop_pair would leave SMs idle, k_hop_pair from
-//    there on.  FP64 tile / pair: 25 / 41 at 128, 33 / 41 at 2048, 58 / 50 at 4096, 545 /
-//    506 at 65536; double-float (true residual) 69 / 77 at 128, 334 / 321 at 65536.
+//    there on.  FP64 tile / pair: 25 / 34 at 128, 33 / 41 at 2048, 56 / 49 at 4096, 531 /
+//    506 at 65536; double-float (true residual) 72 / 75 at 128, 302 / 297 at 65536.
 constexpr int kPairMaxF32 = 32 * 152;
 constexpr int kTileMax = kPairSites * 152;
 inline bool hop_shared_f32(int Vh) { return Vh <= kPairMaxF32; }

@@ -71,11 +71,6 @@ __device__ __forceinline__ double2 cs(double s, double2 a) { return make_double2
 __device__ __forceinline__ double2 axpy_c(double2 a, double2 x, double2 y) {
   return make_double2(fma(-a.y, x.y, fma(a.x, x.x, y.x)), fma(a.y, x.x, fma(a.x, x.y, y.y)));
 }
-__device__ __forceinline__ float4 axpy_c(double2 a, float4 x, float4 y) {
-  const float ar = (float)a.x, ai = (float)a.y;
-  return make_float4(y.x + ar * x.x - ai * x.y, y.y + ar * x.y + ai * x.x, y.z + ar * x.z - ai * x.w,
-                     y.w + ar * x.w + ai * x.z);
-}
 // a x + b y
 __device__ __forceinline__ double2 axpby_c(double2 a, double2 x, double2 b, double2 y) { return axpy_c(a, x, cm(b, y)); }
 __device__ __forceinline__ float4 axpby_c(double2 a, float4 x, double2 b, float4 y) {

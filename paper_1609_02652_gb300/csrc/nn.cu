@@ -514,13 +514,6 @@ __global__ void k_fgcr_start(CGScalars* s, double delta2, double floor_rr) {
   s->iter = 0;
 }
 
-__global__ void k_scale32(float4* x, float a, long n) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    float4 v = x[i];
-    x[i] = make_float4(a * v.x, a * v.y, a * v.z, a * v.w);
-  }
-}
-
 }  // namespace pfmp
 
 using namespace pfmp;

@@ -180,21 +180,6 @@ __host__ __device__ __forceinline__ Mat3<T> matmul_nd(const Mat3<T>& A, const Ma
     }
   return C;
 }
-// A^dag * B
-template <typename T>
-__host__ __device__ __forceinline__ Mat3<T> matmul_dn(const Mat3<T>& A, const Mat3<T>& B) {
-  Mat3<T> C;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      cplx<T> s = cj_mul(A.m[0][i], B.m[0][j]);
-      s = s + cj_mul(A.m[1][i], B.m[1][j]);
-      s = s + cj_mul(A.m[2][i], B.m[2][j]);
-      C.m[i][j] = s;
-    }
-  return C;
-}
 template <typename T>
 __host__ __device__ __forceinline__ Mat3<T> dagger(const Mat3<T>& A) {
   Mat3<T> C;
@@ -202,15 +187,6 @@ __host__ __device__ __forceinline__ Mat3<T> dagger(const Mat3<T>& A) {
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) C.m[i][j] = conj(A.m[j][i]);
-  return C;
-}
-template <typename T>
-__host__ __device__ __forceinline__ Mat3<T> mat_add(const Mat3<T>& A, const Mat3<T>& B) {
-  Mat3<T> C;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) C.m[i][j] = A.m[i][j] + B.m[i][j];
   return C;
 }
 template <typename T>
