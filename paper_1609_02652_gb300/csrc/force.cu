@@ -549,11 +549,12 @@ __device__ __forceinline__ cplx<T> tr_lambda_rt(int a, Get Z) {
 }
 
 // The gauge force, F += (beta/6) Im tr(lambda_a U S), and the clover force,
-// F += (1/16) Re tr(lambda_a [U X - Y U^dag]), one thread per link: FP32 on large lattices.
+// F += (1/16) Re tr(lambda_a [U X - Y U^dag]), one thread per link: FP32 on large lattices, and
+// the FP64 gauge force on all but the smallest.
 // A block takes 32 sites of parity blockIdx.y and warp mu the links U_mu of those sites,
 // so the four warps share the fields they read through L1.
 template <typename T, int KIND>
-__global__ void __launch_bounds__(128, 4) k_leaf_force(double* F, const void* gauge, const cplx<T>* D, Geom g, double coef) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) k_leaf_force(double* F, const void* gauge, const cplx<T>* D, Geom g, double coef) {
   chain_enter();
   const int cb = blockIdx.x * 32 + (threadIdx.x & 31);
   const int mu = threadIdx.x >> 5;
@@ -583,9 +584,9 @@ __global__ void __launch_bounds__(128, 4) k_leaf_force(double* F, const void* ga
   for (int a = 0; a < 8; ++a) fptr(F, g, p, mu, a)[cb] += coef * (double)(KIND == LEAF_GAUGE ? t[a].im : t[a].re);
 }
 
-// The same with 24 threads per site, one per leaf (mu, nu, side), in blocks of 4 sites: FP64
-// (bound by its pipe: equal small pieces for every SM, no thread with a long chain) and FP32
-// on small lattices.  The leaves meet in shared memory; 12 threads per site take one row of
+// The same with 24 threads per site, one per leaf (mu, nu, side), in blocks of 4 sites: the FP64
+// clover force (bound by its pipe: equal small pieces for every SM, no thread with a long
+// chain) and both precisions on small lattices.  The leaves meet in shared memory; 12 threads per site take one row of
 // Z = U X - Y U^dag each, then every thread one or two of the 32 components.
 constexpr int kLeafSites = 4;
 template <typename T, int KIND>
@@ -646,11 +647,24 @@ __global__ void __launch_bounds__(24 * kLeafSites) k_leaf_force_split(double* F,
 // lattices whose links, 128 to a block, leave SMs idle or with one block in flight
 static bool force_small(const Geom& g) { return g.Vh < 32 * 152 * 2; }
 
+// FP64 gauge force: a thread per leaf (k_leaf_force_split) on the smallest lattices, a thread per
+// link from this many sites per parity on.  The leaves' links come in pieces of 4 sites and
+// cross shared memory again, which costs more than the pipe's share of a whole link once
+// there is a block of links for most SMs (us per force, leaf / link: 37 / 62 at 256, 87 / 64 at
+// 1296, 345 / 198 at 7560, 2840 / 1250 at 65536, where a thread per site took 2260).  Clover
+// leaves have four products and 18 more numbers to load each, and stay with a thread per leaf.
+constexpr int kGaugeWhole64 = 768;
+
 template <typename T, int KIND>
 static void leaf_force(pfmp_ctx* c, double* F, const void* gauge, const cplx<T>* D, double coef) {
   const dim3 split(nblocks(c->g.Vh, kLeafSites), 2);
   if constexpr (sizeof(T) == 8) {
-    k_leaf_force_split<T, KIND><<<split, 24 * kLeafSites, 0, c->stream>>>(F, gauge, D, c->g, coef);
+    bool whole = false;
+    if constexpr (KIND == LEAF_GAUGE) whole = c->g.Vh >= kGaugeWhole64;
+    if (whole)
+      k_leaf_force<T, LEAF_GAUGE><<<dim3(nblocks(c->g.Vh, 32), 2), 128, 0, c->stream>>>(F, gauge, D, c->g, coef);
+    else
+      k_leaf_force_split<T, KIND><<<split, 24 * kLeafSites, 0, c->stream>>>(F, gauge, D, c->g, coef);
   } else {
     if (force_small(c->g))
       k_leaf_force_split<T, KIND><<<split, 24 * kLeafSites, 0, c->stream>>>(F, gauge, D, c->g, coef);
