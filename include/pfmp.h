@@ -490,7 +490,9 @@ int pfmp_nn_apply(pfmp_nn* nn, int prec, void* out, const void* in);
  * FP16 operands
  * (inputs scaled by 1 / rms of the network input, weights packed as [[Re, -Im], [Im,
  * Re]]) with FP32 accumulation; training always uses the FP32 kernels.  on = 0 selects
- * the FP32 kernels everywhere.  PFMP_E_UNSUPPORTED if the network has no such layer;
+ * the FP32 kernels everywhere.  PFMP_E_UNSUPPORTED unless every layer is one of these;
+ * PFMP_E_INVALID from pfmp_nn_apply / pfmp_solve_fgcr while it is on for channels that
+ * return to 1 in between (the sequence is 1 -> 8 -> ... -> 8 -> 1);
  * PFMP_E_TIMEOUT from pfmp_nn_apply / pfmp_solve_fgcr if a tensor-core kernel gave up
  * waiting for its MMAs (bounded waits; the context stays usable).                       */
 int pfmp_nn_set_tensor_cores(pfmp_nn* nn, int on);

@@ -12,7 +12,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def _work(dims, stream, out):
+def _drive(dims, stream, out):
     import numpy as np
     import torch
 
@@ -76,7 +76,7 @@ def _main(path):
 
     def run(dims):
         try:
-            _work(dims, torch.cuda.Stream(), out)
+            _drive(dims, torch.cuda.Stream(), out)
         except Exception as e:  # noqa: BLE001
             errors.append(repr(e))
 
