@@ -214,9 +214,9 @@ double fma_rate(pfmp_ctx* c, int prec);
 
 // slots of pfmp_op::graph beyond the CG's (indexed by precision)
 constexpr int kGraphMs64 = 4, kGraphMs32 = 5;
-// replay the chunk that `launch` enqueues on the context's stream as a CUDA graph, captured
-// (on op->cap) when the slot holds another key or chunk length
-void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch);
+// replay the chunk that `launch` makes as a CUDA graph, recorded (LaunchRecord) when the slot
+// holds another key or chunk length
+void run_recorded(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch);
 
 // solver.cu
 int solve(pfmp_op* op, int method, double tol, int max_iter, double delta, int check_every, void* x,

@@ -118,9 +118,9 @@ void launch_site(const HopParams<PREC>& a, int bs, cudaStream_t st) {
   // FP16 storage without a sum needs 127 registers, whether it may have 255 or 128
   constexpr int B2 = PREC == PFMP_F32 || RED ? 2 : 4;
   switch (m) {
-    case 2: k_hop<PREC, DAG, EPI, RED, B2><<<n, bs, 0, st>>>(a); break;
-    case 4: k_hop<PREC, DAG, EPI, RED, 4><<<n, bs, 0, st>>>(a); break;
-    default: k_hop<PREC, DAG, EPI, RED, B><<<n, bs, 0, st>>>(a);
+    case 2: launch_plain(k_hop<PREC, DAG, EPI, RED, B2>, n, bs, st, a); break;
+    case 4: launch_plain(k_hop<PREC, DAG, EPI, RED, 4>, n, bs, st, a); break;
+    default: launch_plain(k_hop<PREC, DAG, EPI, RED, B>, n, bs, st, a);
   }
 }
 
@@ -136,9 +136,9 @@ void launch(const HopParams<PREC>& a, pfmp_op* op) {
     const int ns = split_of<PREC>(op);
     const long n = (long)a.g.Vh * ns;
     switch (ns) {
-      case 2: k_hop_split<PREC, DAG, EPI, RED, 2><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
-      case 4: k_hop_split<PREC, DAG, EPI, RED, 4><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
-      case 8: k_hop_split<PREC, DAG, EPI, RED, 8><<<nblocks(n, bs), bs, 0, c->stream>>>(a); break;
+      case 2: launch_plain(k_hop_split<PREC, DAG, EPI, RED, 2>, nblocks(n, bs), bs, c->stream, a); break;
+      case 4: launch_plain(k_hop_split<PREC, DAG, EPI, RED, 4>, nblocks(n, bs), bs, c->stream, a); break;
+      case 8: launch_plain(k_hop_split<PREC, DAG, EPI, RED, 8>, nblocks(n, bs), bs, c->stream, a); break;
       default:
         if constexpr (PREC == PFMP_F32) {
           if (!hop_shared_f32(a.g.Vh)) {

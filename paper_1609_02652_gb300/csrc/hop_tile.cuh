@@ -422,7 +422,7 @@ void launch_shared(const HopParams<PREC>& a, cudaStream_t st) {
   const int Vh = a.g.Vh;
   if constexpr (PREC != PFMP_F32) {
     if (Vh <= kTileMax) {
-      k_hop_tile<PREC, DAG, EPI, RED><<<nblocks(Vh, kTileSites), 16 * kTileSites, 0, st>>>(a);
+      launch_plain(k_hop_tile<PREC, DAG, EPI, RED>, nblocks(Vh, kTileSites), 16 * kTileSites, st, a);
       return;
     }
   }
@@ -432,7 +432,7 @@ void launch_shared(const HopParams<PREC>& a, cudaStream_t st) {
   if constexpr (PREC == PFMP_F32)
     launch_chained(k_hop_pair<PREC, DAG, EPI, RED>, blocks, 8 * kPairSites, st, a);
   else
-    k_hop_pair<PREC, DAG, EPI, RED><<<blocks, 8 * kPairSites, 0, st>>>(a);
+    launch_plain(k_hop_pair<PREC, DAG, EPI, RED>, blocks, 8 * kPairSites, st, a);
 }
 
 }  // namespace pfmp

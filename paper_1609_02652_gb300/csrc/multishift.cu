@@ -354,7 +354,7 @@ static MSWork& ms_work(pfmp_op* op, int ns, int prec) {
   if (!op->ms) op->ms = new MSWork();
   MSWork& w = *op->ms;
   if (w.cap < ns) {
-    // a captured chunk holds the arrays that are replaced here
+    // a chunk's graph holds the arrays that are replaced here
     for (int g : {kGraphMs64, kGraphMs32})
       if (op->graph[g].exec) {
         cudaGraphExecDestroy(op->graph[g].exec);
@@ -411,10 +411,11 @@ static void ms_chunk(pfmp_op* op, int prec, MSWork& w, void* pseed, void* Ap, lo
 }
 
 // Up to this many sites per parity the kernels of an iteration are shorter than the
-// host takes to launch them, and a chunk is replayed as a CUDA graph (as the CG's).  The graph
-// depends on the workspace only, not on the solve's shifts: solves that alternate between
-// numbers of shifts share it (with a capture for each change of their number a solve of 0.21 ms
-// took 0.35).  A chunk cut short by the iteration cap is launched directly.
+// host takes to launch them, and a chunk is replayed as a CUDA graph (recorded, not captured from
+// a stream: other threads may synchronise the device meanwhile).  The graph depends on the
+// workspace only, not on the solve's shifts: solves that alternate between numbers of shifts
+// share it (with a graph made at each change of their number a solve of 0.21 ms took 0.35).
+// A chunk cut short by the iteration cap is launched directly.
 constexpr int kMsGraphMax = 32768;
 
 // x[k] = (K + sigma_k)^{-1} b in FP64 or FP32 (x, b of precision prec).  Returns the
@@ -491,7 +492,7 @@ int solve_multishift(pfmp_op* op, int prec, int ns, const std::complex<double>* 
     };
     if (c->g.Vh <= kMsGraphMax && !c->prof.on && chunk == check) {
       const void* key[4] = {w.d_sh, w.d_x, w.d_p, w.d_act};
-      run_graph(op, op->graph[prec == PFMP_F64 ? kGraphMs64 : kGraphMs32], key, chunk, launch);
+      run_recorded(op, op->graph[prec == PFMP_F64 ? kGraphMs64 : kGraphMs32], key, chunk, launch);
     } else {
       launch();
     }

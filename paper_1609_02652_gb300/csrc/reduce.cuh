@@ -2,6 +2,9 @@
 // partial per block, and the last block to finish (atomic ticket) adds the partials in
 // a fixed order.  The result therefore does not depend on block scheduling.
 #pragma once
+#include <tuple>
+#include <utility>
+
 #include "pfmp_internal.cuh"
 
 namespace pfmp {
@@ -19,8 +22,8 @@ namespace pfmp {
 // K at 4^3x8 (four launches of k_hop_pair) 16.4 -> 10.7 us.  The FP64 stencils and force
 // contractions gain nothing (the FP64 force at 6x10x14x18 +2%), nor do the one-thread-per-site
 // stencils (K at 32^3x64 +2%): those are launched in the ordinary way.  Inside a CUDA graph
-// these edges cost more than they hide (mixed solve at 16^3x32 6.1 -> 6.9 ms), so a captured
-// launch is an ordinary one; kernels that run on both sides are told (chained) where they can
+// these edges cost more than they hide (mixed solve at 16^3x32 6.1 -> 6.9 ms), so a captured or
+// recorded launch is an ordinary one; kernels that run on both sides are told (chained) where they can
 // be without a cost.
 __device__ __forceinline__ void chain_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -56,14 +59,59 @@ __device__ __forceinline__ double2 ld_live(const double2* p) {
   asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
   return v;
 }
+// A chunk of launches as a CUDA graph, node after node: while a LaunchRecord of this thread is
+// current, launch_plain and launch_chained add to its graph instead of launching.  A stream
+// capture makes the same graph, but a cudaDeviceSynchronize in any other thread fails while a
+// stream captures, and the capture with it.
+struct LaunchRecord {
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t last = nullptr;
+  long long kernels = 0;
+  static LaunchRecord*& current() {
+    static thread_local LaunchRecord* r = nullptr;
+    return r;
+  }
+  LaunchRecord() {
+    PFMP_CUDA(cudaGraphCreate(&graph, 0));
+    current() = this;
+  }
+  LaunchRecord(const LaunchRecord&) = delete;
+  ~LaunchRecord() {
+    current() = nullptr;
+    cudaGraphDestroy(graph);
+  }
+  template <typename... P, size_t... I>
+  void add(void (*kernel)(P...), dim3 grid, dim3 block, std::tuple<P...> args, std::index_sequence<I...>) {
+    void* at[] = {(void*)&std::get<I>(args)...};
+    cudaKernelNodeParams p{};
+    p.func = (void*)kernel;
+    p.gridDim = grid;
+    p.blockDim = block;
+    p.kernelParams = at;
+    cudaGraphNode_t node;
+    PFMP_CUDA(cudaGraphAddKernelNode(&node, graph, &last, last ? 1 : 0, &p));
+    last = node;
+    ++kernels;
+  }
+};
+template <typename... P, typename... A>
+void launch_plain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  if (LaunchRecord* r = LaunchRecord::current())
+    r->add(kernel, grid, block, std::tuple<P...>(static_cast<P>(args)...), std::index_sequence_for<P...>());
+  else
+    kernel<<<grid, block, 0, st>>>(static_cast<P>(args)...);
+}
+
 // whether launches on st are chained
 inline bool chain_launches(cudaStream_t st) {
+  if (LaunchRecord::current()) return false;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   PFMP_CUDA(cudaStreamIsCapturing(st, &capture));
   return capture == cudaStreamCaptureStatusNone;
 }
 template <typename... P, typename... A>
 void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  if (LaunchRecord::current()) return launch_plain(kernel, grid, block, st, args...);
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;

@@ -82,18 +82,44 @@ static void launch_chunk(pfmp_op* op, int prec, void* x, void* r, void* p, void*
   }
 }
 
-// A chunk of iterations, captured once into a CUDA graph (all parameters fixed: the scalars
-// live on the device) and replayed on the context's stream, which removes the per-launch
-// host cost.
-void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch) {
-  pfmp_ctx* c = op->ctx;
+// whether G is the graph of this key and chunk length; if not, it is dropped
+static bool graph_is(pfmp_op::Graph& G, const void* const key[4], int chunk) {
   bool hit = G.exec && G.chunk == chunk;
   for (int k = 0; k < 4 && hit; ++k) hit = G.key[k] == key[k];
-  if (!hit) {
-    if (G.exec) {
-      cudaGraphExecDestroy(G.exec);
-      G.exec = nullptr;
-    }
+  if (!hit && G.exec) {
+    cudaGraphExecDestroy(G.exec);
+    G.exec = nullptr;
+  }
+  return hit;
+}
+static void graph_set(pfmp_op::Graph& G, cudaGraph_t graph, const void* const key[4], int chunk, long long kernels) {
+  PFMP_CUDA(cudaGraphInstantiate(&G.exec, graph, 0));
+  G.chunk = chunk;
+  G.kernels = kernels;
+  for (int k = 0; k < 4; ++k) G.key[k] = key[k];
+}
+
+// A chunk of iterations as a CUDA graph (all parameters fixed: the scalars live on the
+// device), made once and replayed on the context's stream, which removes the per-launch host
+// cost: recorded, where every launch of the chunk is a launch_plain or launch_chained, ...
+void run_recorded(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk, const std::function<void()>& launch) {
+  if (!graph_is(G, key, chunk)) {
+    const long long kapply0 = op->kapply;
+    LaunchRecord r;
+    launch();
+    op->kapply = kapply0;
+    count_launches(-r.kernels);  // recorded, not launched
+    graph_set(G, r.graph, key, chunk, r.kernels);
+  }
+  PFMP_CUDA(cudaGraphLaunch(G.exec, op->ctx->stream));
+  count_launches(G.kernels);
+}
+
+// ... or captured from a stream
+static void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chunk,
+                      const std::function<void()>& launch) {
+  pfmp_ctx* c = op->ctx;
+  if (!graph_is(G, key, chunk)) {
     if (!op->cap) PFMP_CUDA(cudaStreamCreateWithFlags(&op->cap, cudaStreamNonBlocking));
     cudaStream_t keep = c->stream;
     cudaGraph_t graph = nullptr;
@@ -111,14 +137,16 @@ void run_graph(pfmp_op* op, pfmp_op::Graph& G, const void* const key[4], int chu
     }
     c->stream = keep;
     op->kapply = kapply0;
-    G.kernels = launch_count() - n0;
-    count_launches(-G.kernels);  // captured, not launched
+    const long long kernels = launch_count() - n0;
+    count_launches(-kernels);  // captured, not launched
     PFMP_CUDA(cudaStreamEndCapture(op->cap, &graph));
-    cudaError_t e = cudaGraphInstantiate(&G.exec, graph, 0);
+    try {
+      graph_set(G, graph, key, chunk, kernels);
+    } catch (...) {
+      cudaGraphDestroy(graph);
+      throw;
+    }
     cudaGraphDestroy(graph);
-    PFMP_CUDA(e);
-    G.chunk = chunk;
-    for (int k = 0; k < 4; ++k) G.key[k] = key[k];
   }
   PFMP_CUDA(cudaGraphLaunch(G.exec, c->stream));
   count_launches(G.kernels);

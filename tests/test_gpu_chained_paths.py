@@ -18,6 +18,10 @@ def _drive(dims, stream, out):
 
     from paper_1609_02652_gb300 import capi
 
+    def wait():  # not the device: a solve of the other thread may be capturing its chunk
+        torch.cuda.current_stream().synchronize()
+        stream.synchronize()
+
     V = dims[0] * dims[1] * dims[2] * dims[3]
     gen = torch.Generator(device="cuda").manual_seed(11)
     h = [torch.randn(V, 4, 8, generator=gen, dtype=torch.float64, device="cuda") for _ in range(3)]
@@ -26,13 +30,13 @@ def _drive(dims, stream, out):
     n = capi.pfmp_spinor_bytes(ctx, capi.PFMP_F32) // 4
     b = torch.randn(n, generator=gen, dtype=torch.float32, device="cuda")
     b64 = torch.randn(n, generator=gen, dtype=torch.float64, device="cuda")
-    torch.cuda.synchronize()
+    wait()
     capi.pfmp_gauge_from_algebra(ctx, h[0], 0.4, capi.PFMP_DEVICE)
     op = capi.pfmp_op_create(ctx, 0.12, 1.0)
     xs = [torch.zeros_like(b) for _ in range(3)]
     v = [b.clone(), torch.zeros_like(b)]
     x = torch.zeros_like(b64)
-    torch.cuda.synchronize()
+    wait()
     capi.pfmp_solve_multishift_prec(op, capi.PFMP_F32, np.array([0.0, 0.3 + 0.4j, 1.5 - 0.2j]), xs, b, 1e-6, 200)
     for k in range(8):
         capi.pfmp_kop(op, capi.PFMP_F32, v[(k + 1) & 1], v[k & 1])
@@ -53,13 +57,13 @@ def _drive(dims, stream, out):
         capi.pfmp_action_refresh(A)
         for term in range(5):
             F = torch.zeros(V, 4, 8, dtype=torch.float64, device="cuda")
-            torch.cuda.synchronize()
+            wait()
             capi.pfmp_action_force(A, term, F, capi.PFMP_DEVICE)
             forces.append(F)
     T, S = capi.pfmp_schedule_2mn(1, 0.05, 0.19)
     P = h[2]
     capi.pfmp_md(A, T, np.array([S]), [0] * 5, P, capi.PFMP_DEVICE)
-    torch.cuda.synchronize()
+    wait()
     for i, t in enumerate(xs + [v[0], x] + forces + [P]):
         out[f"{'x'.join(map(str, dims))}_{i}"] = t.cpu().numpy()
     capi.pfmp_action_destroy(A)
